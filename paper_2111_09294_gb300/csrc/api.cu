@@ -343,7 +343,7 @@ struct PlainPath {
             launch_block_apply<double>(L.J, r, y, c->partials, sc, st);
             c->launches++;
         } else {
-            launch_update<double>(L.N, u, r, p, q, y, mode, c->partials, sc, st);
+            launch_update(L.N, u, r, p, q, y, mode, c->partials, sc, st);
         }
     }
     void restrict_(const double *a, const double *b, int withW, double *zr, Scalars *sc) {
@@ -1970,35 +1970,36 @@ xdcg_status setup_impl(xdcg_ctx *c, const xdcg_matrix *K, const xdcg_deflation *
 
     // W = K Z and E = Z^T W
     int *d_extBox = upload_tmp(c, extBox), *d_extNode = upload(c, extNode);
-    int *d_extPtr = upload(c, extPtr), *d_ownPtr = upload(c, ownPtr), *d_own = upload(c, ownNodes);
+    int *d_ownPtr = upload(c, ownPtr), *d_own = upload(c, ownNodes);
     long long *d_wOff = upload(c, wOff);
     double *d_W = dalloc<double>(c, nW);
-    if (!d_extBox || !d_extNode || !d_extPtr || !d_ownPtr || !d_own || !d_wOff || !d_W)
+    if (!d_extBox || !d_extNode || !d_ownPtr || !d_own || !d_wOff || !d_W)
         return XDCG_OOM;
     // Z by value: the caller's blocks for the set-up kernels (node order) and,
     // in box order, for the FP64 restriction and prolongation
     ZvalDev zv{nullptr, nullptr};
     double *d_zslot = nullptr;
+    std::vector<long long> zslotOffs;
     long long *d_zslotOff = nullptr;
     if (valued) {
         zv.v = upload_tmp(c, zval);
         zv.off = upload_tmp(c, zvOff);
         std::vector<double> zslot;
-        std::vector<long long> zslotOff(N);
+        zslotOffs.resize(N);
         zslot.reserve(zval.size());
         for (int t = 0; t < N; ++t) {
             const int I = ownNodes[t];
-            zslotOff[t] = (long long)zslot.size();
+            zslotOffs[t] = (long long)zslot.size();
             zslot.insert(zslot.end(), zval.begin() + zvOff[I], zval.begin() + zvOff[I + 1]);
         }
         d_zslot = upload(c, zslot);
-        d_zslotOff = upload(c, zslotOff);
+        d_zslotOff = upload(c, zslotOffs);
         if (!zv.v || !zv.off || !d_zslot || !d_zslotOff) return XDCG_OOM;
     }
     launch_build_W(kin, nExt, d_extBox, d_extNode, d_wOff, d_sub, d_x64, d_hs, d_menr, zv, d_W,
                    st);
     // node data in box order (slots) and per-entry dof data for the box kernels
-    std::vector<int> ownDof(N), extDof(nExt);
+    std::vector<int> ownDof(N);
     std::vector<unsigned char> ownB(N), extB(nExt);
     std::vector<signed char> ownH(N);
     std::vector<double> ownCoords(3 * (size_t)N);
@@ -2011,11 +2012,48 @@ xdcg_status setup_impl(xdcg_ctx *c, const xdcg_matrix *K, const xdcg_deflation *
         ownSub[t] = sub[I];
         for (int e = 0; e < 3; ++e) ownCoords[3 * (size_t)t + e] = coords[3 * (size_t)I + e];
     }
-    for (int e = 0; e < nExt; ++e) {
-        extDof[e] = dof[extNode[e]];
-        extB[e] = (unsigned char)kindb[extNode[e]];
-    }
-    int *d_ownDof = upload(c, ownDof), *d_extDof = upload(c, extDof);
+    for (int e = 0; e < nExt; ++e) extB[e] = (unsigned char)kindb[extNode[e]];
+    // the FP64 restriction's work lists (GrpList): each box's items (node,
+    // first entry of its block) dealt to the slots in turn, three rows a record
+    auto build_groups = [&](const std::vector<int> &ptr, const std::vector<int> &node,
+                            const std::vector<long long> &off, GrpList &G) -> bool {
+        std::vector<long long> gp(S + 1, 0);
+        for (int s = 0; s < S; ++s) {
+            const int slots = box_slots(menr[s] ? 12 : 6);
+            std::vector<int> len(slots, 0);
+            for (int e = ptr[s]; e < ptr[s + 1]; ++e)
+                len[(e - ptr[s]) % slots] += kindb[node[e]] / 3;
+            gp[s + 1] = gp[s] + (long long)slots * *std::max_element(len.begin(), len.end());
+        }
+        std::vector<int2> rec((size_t)gp[S], make_int2(0, -1));
+        for (int s = 0; s < S; ++s) {
+            const int M = menr[s] ? 12 : 6, slots = box_slots(M);
+            std::vector<int> len(slots, 0);
+            for (int e = ptr[s]; e < ptr[s + 1]; ++e) {
+                const int q = (e - ptr[s]) % slots, I = node[e];
+                for (int ci = 0; ci < kindb[I] / 3; ++ci)
+                    rec[gp[s] + q + (long long)slots * len[q]++] =
+                        make_int2((int)((off[e] + 3LL * ci * M) / 6), dof[I] + 3 * ci);
+            }
+        }
+        G.ptr = upload(c, gp);
+        G.rec = upload(c, rec);
+        return G.ptr && G.rec;
+    };
+    GrpList gOwn{nullptr, nullptr}, gExt{nullptr, nullptr};
+    if (!build_groups(extPtr, extNode, wOff, gExt)) return XDCG_OOM;
+    if (valued && !build_groups(ownPtr, ownNodes, zslotOffs, gOwn)) return XDCG_OOM;
+    // its units, the ones with the most coupled rows first
+    std::vector<int2> units;
+    for (int s = 0; s < S; ++s)
+        for (int h = 0; h < (menr[s] ? 2 : 1); ++h) units.push_back(make_int2(s, h));
+    std::stable_sort(units.begin(), units.end(), [&](const int2 &x, const int2 &y) {
+        auto chain = [&](int s) { return (extPtr[s + 1] - extPtr[s]) / box_slots(menr[s] ? 12 : 6); };
+        return chain(x.x) > chain(y.x);
+    });
+    const int2 *d_units = upload(c, units);
+    if (!d_units) return XDCG_OOM;
+    int *d_ownDof = upload(c, ownDof);
     unsigned char *d_ownB = upload(c, ownB), *d_extB = upload(c, extB);
     signed char *d_ownH = upload(c, ownH);
     double *d_ownX = dalloc<double>(c, 3 * (size_t)N);
@@ -2025,9 +2063,12 @@ xdcg_status setup_impl(xdcg_ctx *c, const xdcg_matrix *K, const xdcg_deflation *
         if (!d_oc || !d_centre2 || !d_os) return XDCG_OOM;
         if (d_ownX) launch_xrel(N, d_oc, d_centre2, d_os, d_ownX, nullptr, st);
     }
-    if (!d_ownDof || !d_extDof || !d_ownB || !d_extB || !d_ownH || !d_ownX) return XDCG_OOM;
+    if (!d_ownDof || !d_ownB || !d_extB || !d_ownH || !d_ownX) return XDCG_OOM;
     auto &B64 = c->L64.B;
     B64.nBox = S;
+    B64.nOwn = N;
+    B64.nUnits = (int)units.size();
+    B64.unit = d_units;
     B64.col0 = d_col0;
     B64.menr = d_menr;
     B64.ownPtr = d_ownPtr;
@@ -2037,10 +2078,8 @@ xdcg_status setup_impl(xdcg_ctx *c, const xdcg_matrix *K, const xdcg_deflation *
     B64.ownX = d_ownX;
     B64.ownZ = d_zslotOff;
     B64.Zt = d_zslot;
-    B64.extPtr = d_extPtr;
-    B64.extDof = d_extDof;
-    B64.extB = d_extB;
-    B64.wOff = d_wOff;
+    B64.own = gOwn;
+    B64.ext = gExt;
     B64.W = d_W;
     c->Einv = dalloc<double>(c, (size_t)k * k);
     c->E = dalloc<double>(c, (size_t)k * k);

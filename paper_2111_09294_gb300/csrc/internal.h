@@ -144,26 +144,36 @@ struct NodeDev {
     const int *menr;          // [nBox] 1 if the box carries enriched modes
 };
 
-// Box-level data, node data in box order ("slots": the nodes of box s are
-// slots ownPtr[s] .. ownPtr[s+1]-1), and the W entries of each box (nodes
-// coupled to the box, W block b_I x M_s row-major at wOff[e]).  Z is
-// matrix-free (ownX, ownH) in the FP64 path and explicit (Zt at ownZ[t],
-// b_I x M_s row-major) in the block-scaled FP32 path.
+// Slots of a box's FP64 restriction: every box_slots(M)-th node is one slot's
+// chain (M coarse columns per box).
+__host__ __device__ constexpr int box_slots(int M) { return 4 * (32 / M); }
+
+// The restriction's work lists: box s's records rec[ptr[s] .. ptr[s+1]), slot
+// q's chain at every box_slots(M)-th record from q on (padded with y = -1 to a
+// common length).  A record is three rows of one node: their block of W (or of
+// Z by value), 3 x M row-major, at 6 x, and their first dof y.
+struct GrpList {
+    const long long *ptr;         // [nBox + 1]
+    const int2 *rec;
+};
+
+// Box-level data of the FP64 path, node data in box order ("slots": the nodes
+// of box s are slots ownPtr[s] .. ownPtr[s+1]-1), and the W entries of each
+// box (nodes coupled to the box, W block b_I x M_s row-major).  Z is
+// matrix-free (ownX, ownH) or by value (Zt at ownZ[t], b_I x M_s row-major).
 template <typename T>
 struct BoxDev {
-    int nBox;
+    int nBox, nOwn, nUnits;
     const int *col0, *menr;       // first coarse column / enriched-mode flag per box
+    const int2 *unit;             // [nUnits] restriction units: box, its first or second six columns
     const int *ownPtr;            // [nBox + 1]
     const int *ownDof;            // [slots] first dof of the node
     const unsigned char *ownB;    // [slots] dofs of the node (3, 6, 15)
     const signed char *ownH;      // [slots] H(x_I)
     const T *ownX;                // [3 slots] position relative to the box centre
-    const long long *ownZ;        // [slots] offset of the explicit Z~ block
-    const T *Zt;                  // explicit Z~ (scaled path only)
-    const int *extPtr;            // [nBox + 1]
-    const int *extDof;            // [entries] first dof of the entry's node
-    const unsigned char *extB;    // [entries] dofs of the entry's node
-    const long long *wOff;        // [entries]
+    const long long *ownZ;        // [slots] offset of the node's block of Z by value
+    const T *Zt;                  // Z by value, else null
+    GrpList own, ext;             // rows of Zt (Z by value only) and of W
     const T *W;
 };
 
@@ -183,9 +193,9 @@ int spmv_persistent_grid(int nSlicesTotal, int shape);
 template <typename T>
 int spmv_shape_count();
 
-template <typename T>
-void launch_update(const NodeDev<T> &N, T *u, T *r, const T *p, const T *q, T *y, int mode,
-                   double *partials, Scalars *sc, cudaStream_t st);
+void launch_update(const NodeDev<double> &N, double *u, double *r, const double *p,
+                   const double *q, double *y, int mode, double *partials, Scalars *sc,
+                   cudaStream_t st);
 
 // Row-parallel form of the block-scaled FP32 path: per box, the rows of its
 // own nodes (Z~, column-major: column c of box s at Z + zBase[s] + c * R_s;

@@ -3,6 +3,8 @@
 // Cholesky factors (Algorithm 3, first step; blocks of Eqs. block_jacobi /
 // block_jacobi_enr) and the partial sums ||r||^2, r^T y; and the set-up
 // factorisation of the node blocks.
+#include <algorithm>
+
 #include "reduce.cuh"
 
 namespace xdcg {
@@ -11,117 +13,206 @@ namespace xdcg {
 
 __host__ __device__ constexpr int tri(int i, int j) { return i * (i + 1) / 2 + j; }
 
-template <typename T, int B>
-__device__ __forceinline__ void update_node(const T *__restrict__ L, int cnt, int t,
-                                            long long d0, T *u, T *r, const T *p, const T *q,
-                                            T *y, int mode, T alpha, double &rr, double &ry) {
-    T w[B];
+// The node's entries are all loaded before anything is stored (u, r and y never
+// overlap p, q or the factors, but the compiler cannot know), so a thread pays
+// one memory round trip instead of one per entry; the factor Lf came earlier
+// still, before the wait for the previous kernel.
+template <int B>
+__device__ __forceinline__ void update_node(const double (&Lf)[B * (B + 1) / 2], long long d0,
+                                            double *u, double *r, const double *p,
+                                            const double *q, double *y, int mode,
+                                            const Scalars *sc, double &rr, double &ry) {
+    double w[B];
 #pragma unroll
     for (int i = 0; i < B; ++i) w[i] = r[d0 + i];
     if (mode == 0) {
+        double uv[B], pv[B], qv[B];
 #pragma unroll
         for (int i = 0; i < B; ++i) {
-            u[d0 + i] = fma(alpha, p[d0 + i], u[d0 + i]);
-            w[i] = fma(-alpha, q[d0 + i], w[i]);
+            uv[i] = u[d0 + i];
+            pv[i] = p[d0 + i];
+            qv[i] = q[d0 + i];
+        }
+        const double alpha = sc->alpha;
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            u[d0 + i] = fma(alpha, pv[i], uv[i]);
+            w[i] = fma(-alpha, qv[i], w[i]);
             r[d0 + i] = w[i];
         }
     }
-    T rv[B];
+    double rv[B];
 #pragma unroll
     for (int i = 0; i < B; ++i) rv[i] = w[i];
     // L w = r (forward), then L^T y = w (backward); diagonal stored inverted
 #pragma unroll
     for (int i = 0; i < B; ++i) {
-        T s = w[i];
+        double s = w[i];
 #pragma unroll
-        for (int j = 0; j < i; ++j) s = fma(-L[(size_t)tri(i, j) * cnt + t], w[j], s);
-        w[i] = s * L[(size_t)tri(i, i) * cnt + t];
+        for (int j = 0; j < i; ++j) s = fma(-Lf[tri(i, j)], w[j], s);
+        w[i] = s * Lf[tri(i, i)];
     }
 #pragma unroll
     for (int i = B - 1; i >= 0; --i) {
-        T s = w[i];
+        double s = w[i];
 #pragma unroll
-        for (int j = i + 1; j < B; ++j) s = fma(-L[(size_t)tri(j, i) * cnt + t], w[j], s);
-        w[i] = s * L[(size_t)tri(i, i) * cnt + t];
+        for (int j = i + 1; j < B; ++j) s = fma(-Lf[tri(j, i)], w[j], s);
+        w[i] = s * Lf[tri(i, i)];
     }
 #pragma unroll
     for (int i = 0; i < B; ++i) {
         y[d0 + i] = w[i];
-        rr += (double)rv[i] * (double)rv[i];
-        ry += (double)rv[i] * (double)w[i];
+        rr += rv[i] * rv[i];
+        ry += rv[i] * w[i];
     }
 }
 
-// Branch-enriched node (15 dofs): one warp per node, lane i holds dof i;
-// each solved entry of the forward and backward substitutions is broadcast
-// by a shuffle, so no thread keeps the whole block in registers.
-template <typename T>
-__device__ __forceinline__ void update_tip_warp(const T *__restrict__ L, int cnt, int t,
-                                                long long d0, T *u, T *r, const T *p,
-                                                const T *q, T *y, int mode, T alpha, double &rr,
-                                                double &ry) {
+// Branch-enriched node (15 dofs): half a warp per node, lane i of the half
+// holds dof i; each solved entry of the forward and backward substitutions is
+// broadcast by a shuffle, so no thread keeps the whole block in registers.
+// The lane's factor row (Lr) and column (Lc) come from before the wait.  Two
+// nodes share a warp because the substitutions are FP64 instructions, which
+// cost the same whether 15 or 30 lanes use them.
+__device__ __forceinline__ void update_tip_half(const double (&Lr)[15], const double (&Lc)[15],
+                                                double dinv, bool act, int lane, long long d0,
+                                                double *u, double *r, const double *p,
+                                                const double *q, double *y, int mode,
+                                                const Scalars *sc, double &rr, double &ry) {
     constexpr int B = 15;
-    const int lane = threadIdx.x & 31;
-    const bool act = lane < B;
-    T ri = T(0);
+    double ri = 0.0;
     if (act) {
         ri = r[d0 + lane];
         if (mode == 0) {
-            u[d0 + lane] = fma(alpha, p[d0 + lane], u[d0 + lane]);
-            ri = fma(-alpha, q[d0 + lane], ri);
+            const double uv = u[d0 + lane], pv = p[d0 + lane], qv = q[d0 + lane];
+            const double alpha = sc->alpha;
+            u[d0 + lane] = fma(alpha, pv, uv);
+            ri = fma(-alpha, qv, ri);
             r[d0 + lane] = ri;
         }
     }
-    const T dinv = act ? L[(size_t)tri(lane, lane) * cnt + t] : T(0);
-    T acc = T(0), w = T(0);
+    double acc = 0.0, w = 0.0;
 #pragma unroll
     for (int j = 0; j < B; ++j) {
-        const T wj = __shfl_sync(0xffffffffu, (ri - acc) * dinv, j);
+        const double wj = __shfl_sync(0xffffffffu, (ri - acc) * dinv, j, 16);
         if (lane == j) w = wj;
-        if (act && lane > j) acc = fma(L[(size_t)tri(lane, j) * cnt + t], wj, acc);
+        if (lane > j) acc = fma(Lr[j], wj, acc);
     }
-    T yv = T(0);
-    T acc2 = T(0);
+    double yv = 0.0, acc2 = 0.0;
 #pragma unroll
     for (int i = B - 1; i >= 0; --i) {
-        const T yi = __shfl_sync(0xffffffffu, (w - acc2) * dinv, i);
+        const double yi = __shfl_sync(0xffffffffu, (w - acc2) * dinv, i, 16);
         if (lane == i) yv = yi;
-        if (act && lane < i) acc2 = fma(L[(size_t)tri(i, lane) * cnt + t], yi, acc2);
+        if (lane < i) acc2 = fma(Lc[i], yi, acc2);
     }
     if (act) {
         y[d0 + lane] = yv;
-        rr += (double)ri * (double)ri;
-        ry += (double)ri * (double)yv;
+        rr += ri * ri;
+        ry += ri * yv;
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-k_update(NodeDev<T> N, T *u, T *r, const T *p, const T *q, T *y, int mode, int nb3, int nb6,
-         double *partials, Scalars *sc) {
-    pdl_wait();
-    if (sc->done != kRunning) return;
-    const T alpha = (T)sc->alpha;
+// Partial sums (||r||^2, r^T y) come in units of kWarps warps' work: 256 nodes
+// of 3 or 6 dofs (one block), or 8 nodes of 15 dofs (half a block, one node
+// per half-warp).  Each unit's two sums are the tree over its lanes and then
+// its 8 warps (or nodes); the two values share the shuffles and FP64 adds of
+// a tree (they are exchanged at its first step, one half-warp keeping each),
+// because FP64 instructions are what these trees cost.
+//
+// Bound by FP64 issue and memory latency: everything that set-up fixed (node
+// lists, factors) is loaded before the wait for the product, everything else
+// in one round trip after it.  48^3 (373k dofs, 115k nodes, 1,932 of them with
+// 15 dofs): 44.9 us before, 28.3 now; 8.9k dofs: 17.4 before, 16.7 now
+// (event-timed in the solve, as all figures of this kernel).
+__global__ void __launch_bounds__(kThreads, 3)
+k_update(NodeDev<double> N, double *u, double *r, const double *p, const double *q, double *y,
+         int mode, int nb3, int nb6, int nUnits, double *partials, Scalars *sc) {
+    // the 15-dof nodes' blocks, whose substitutions take longest, are
+    // scheduled first; their units come last in the sums
+    const int nb15 = (int)gridDim.x - nb3 - nb6;
+    const int bid = (int)blockIdx.x < nb15 ? nb3 + nb6 + (int)blockIdx.x : (int)blockIdx.x - nb15;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double v[2] = {0.0, 0.0};
-    const int bid = blockIdx.x;
-    if (bid < nb3) {
-        const int t = bid * kThreads + threadIdx.x;
-        if (t < N.nStd)
-            update_node<T, 3>(N.Lstd, N.nStd, t, N.dofStart[N.stdNodes[t]], u, r, p, q, y, mode,
-                              alpha, v[0], v[1]);
-    } else if (bid < nb3 + nb6) {
-        const int t = (bid - nb3) * kThreads + threadIdx.x;
-        if (t < N.nH)
-            update_node<T, 6>(N.Lh, N.nH, t, N.dofStart[N.hNodes[t]], u, r, p, q, y, mode,
-                              alpha, v[0], v[1]);
+    __shared__ double sums[2][2 * kWarps];
+    const bool tips = bid >= nb3 + nb6;
+    if (!tips) {
+        if (bid < nb3) {
+            const int t = bid * kThreads + threadIdx.x;
+            const bool act = t < N.nStd;
+            long long d0 = 0;
+            double Lf[6];
+            if (act) {
+                d0 = N.dofStart[N.stdNodes[t]];
+#pragma unroll
+                for (int e = 0; e < 6; ++e) Lf[e] = N.Lstd[(size_t)e * N.nStd + t];
+            }
+            pdl_wait();
+            if (sc->done != kRunning) return;
+            if (act) update_node<3>(Lf, d0, u, r, p, q, y, mode, sc, v[0], v[1]);
+        } else {
+            const int t = (bid - nb3) * kThreads + threadIdx.x;
+            const bool act = t < N.nH;
+            long long d0 = 0;
+            double Lf[21];
+            if (act) {
+                d0 = N.dofStart[N.hNodes[t]];
+#pragma unroll
+                for (int e = 0; e < 21; ++e) Lf[e] = N.Lh[(size_t)e * N.nH + t];
+            }
+            pdl_wait();
+            if (sc->done != kRunning) return;
+            if (act) update_node<6>(Lf, d0, u, r, p, q, y, mode, sc, v[0], v[1]);
+        }
+        // lanes 0-15 keep ||r||^2, lanes 16-31 r^T y
+        const bool hi = lane >= 16;
+        double s = (hi ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[1], 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((lane & 15) == 0) sums[lane >> 4][warp] = s;
     } else {
-        const int t = (bid - nb3 - nb6) * kWarps + (threadIdx.x >> 5);
-        if (t < N.nT)
-            update_tip_warp<T>(N.Lt, N.nT, t, N.dofStart[N.tNodes[t]], u, r, p, q, y, mode,
-                               alpha, v[0], v[1]);
+        const int hl = lane & 15, hw = 2 * warp + (lane >> 4);
+        const int t = (bid - nb3 - nb6) * 2 * kWarps + hw;
+        const bool act = hl < 15 && t < N.nT;
+        long long d0 = 0;
+        double Lr[15], Lc[15], dinv = 0.0;
+        if (t < N.nT) d0 = N.dofStart[N.tNodes[t]];
+#pragma unroll
+        for (int j = 0; j < 15; ++j) {
+            Lr[j] = act && hl > j ? N.Lt[(size_t)tri(hl, j) * N.nT + t] : 0.0;
+            Lc[j] = act && hl < j ? N.Lt[(size_t)tri(j, hl) * N.nT + t] : 0.0;
+        }
+        if (act) dinv = N.Lt[(size_t)tri(hl, hl) * N.nT + t];
+        pdl_wait();
+        if (sc->done != kRunning) return;
+        update_tip_half(Lr, Lc, dinv, act, hl, d0, u, r, p, q, y, mode, sc, v[0], v[1]);
+        // lanes 0-7 of a half-warp keep ||r||^2, lanes 8-15 r^T y
+        const bool hi = (lane & 8) != 0;
+        double s = (hi ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[1], 8);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((lane & 7) == 0) sums[(lane >> 3) & 1][hw] = s;
     }
+    __shared__ bool last;
+    __syncthreads();
+    if (warp == 0) {
+        // lane = 16 (unit of the block) + 8 (value) + warp or node of the unit
+        const int val = (lane >> 3) & 1, un = lane >> 4;
+        double s = un == 0 || tips ? sums[val][8 * un + (lane & 7)] : 0.0;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        const int unit = tips ? nb3 + nb6 + 2 * (bid - nb3 - nb6) + un : bid;
+        if ((lane & 7) == 0 && (un == 0 || tips) && unit < nUnits) {
+            partials[(size_t)val * nUnits + unit] = s;
+            __threadfence();
+        }
+        __syncwarp();
+        if (lane == 0) last = atomicAdd(&sc->ticket[2], 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     double tot[2];
-    if (grid_sum<double, 2>(v, partials, &sc->ticket[2], tot) && threadIdx.x == 0) {
+    sum_partials<2>(partials, &sc->ticket[2], tot, nUnits);
+    if (threadIdx.x == 0) {
         sc->ry = tot[1];
         sc->rr = tot[0];
         if (sc->hist && sc->its < sc->histCap) sc->hist[sc->its] = tot[0];
@@ -136,20 +227,14 @@ k_update(NodeDev<T> N, T *u, T *r, const T *p, const T *q, T *y, int mode, int n
 
 static inline int cdiv(long long a, int b) { return (int)((a + b - 1) / b); }
 
-template <typename T>
-void launch_update(const NodeDev<T> &N, T *u, T *r, const T *p, const T *q, T *y, int mode,
-                   double *partials, Scalars *sc, cudaStream_t st) {
-    const int nb3 = cdiv(N.nStd, kThreads), nb6 = cdiv(N.nH, kThreads),
-              nb15 = cdiv(N.nT, kWarps);
-    int grid = nb3 + nb6 + nb15;
-    if (grid == 0) grid = 1;
-    launch_pdl(k_update<T>, grid, kThreads, 0, st, N, u, r, p, q, y, mode, nb3, nb6, partials, sc);
+void launch_update(const NodeDev<double> &N, double *u, double *r, const double *p,
+                   const double *q, double *y, int mode, double *partials, Scalars *sc,
+                   cudaStream_t st) {
+    const int nb3 = cdiv(N.nStd, kThreads), nb6 = cdiv(N.nH, kThreads), nu15 = cdiv(N.nT, kWarps);
+    const int grid = std::max(nb3 + nb6 + (nu15 + 1) / 2, 1);
+    launch_pdl(k_update, grid, kThreads, 0, st, N, u, r, p, q, y, mode, nb3, nb6,
+               std::max(nb3 + nb6 + nu15, 1), partials, sc);
 }
-template void launch_update<double>(const NodeDev<double> &, double *, double *, const double *,
-                                    const double *, double *, int, double *, Scalars *,
-                                    cudaStream_t);
-template void launch_update<float>(const NodeDev<float> &, float *, float *, const float *,
-                                   const float *, float *, int, double *, Scalars *, cudaStream_t);
 
 // ---- set-up: node-block Cholesky (FP64) ------------------------------------
 

@@ -1,0 +1,41 @@
+"""The FP64 restriction, prolongation and node update over box sizes: one box
+holding every node (its work lists span several staged chunks), boxes of odd
+and unequal sizes, Z from the geometry and by value, with and without the
+enriched modes.  One application of Algorithm 3 against the oracle's; the
+tolerance is the preconditioner's (block condition numbers up to ~1e8 times
+the FP64 round-off)."""
+import numpy as np
+import pytest
+import torch
+
+import xfem_inputs as X
+from oracle import adef2 as O
+from xfem_inputs import cracks as C
+
+pytestmark = pytest.mark.gpu
+
+# m hexes per axis, boxes per axis: 180 nodes in one box; 990 nodes (5 chunks of
+# own nodes, 2 of coupled ones); 7^3 + 6^3-node boxes; a box with one layer
+SIZES = [(5, 1), (9, 1), (13, 2), (7, 3)]
+
+
+@pytest.mark.parametrize("m,n_box", SIZES)
+@pytest.mark.parametrize("form", ["enriched", "rigid", "valued"])
+def test_precond_box_sizes(m, n_box, form):
+    from paper_2111_09294_gb300 import Solver
+    P = X.build_problem(m, [C.PlanarEdgeCrack(0.5, 0.41, 1.25 / m)], n_box)
+    K, M, Co = O.setup(P, enriched_modes=form != "rigid")
+    kw = {}
+    if form == "valued":
+        Z, col0 = O.deflation_basis(P)
+        Z = Z.tocsr()
+        dof, sub = P.dof_ptr, P.sub_of_node
+        kw = dict(z_cols=np.diff(col0).astype(np.int32), z_values=np.concatenate(
+            [Z[dof[i]:dof[i + 1], col0[sub[i]]:col0[sub[i] + 1]].toarray().ravel()
+             for i in range(P.n_nodes)]))
+    s = Solver.from_problem(P, enriched_modes=form != "rigid", **kw)
+    r = np.random.default_rng(m).standard_normal(P.n)
+    z = s.precond(torch.tensor(r, device="cuda")).cpu().numpy()
+    ref = O.adef2_apply(K, M, Co, r)
+    assert np.linalg.norm(z - ref) <= 1e-8 * np.linalg.norm(ref)
+    s.close()

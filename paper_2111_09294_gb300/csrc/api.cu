@@ -2309,6 +2309,7 @@ xdcg_status setup_impl(xdcg_ctx *c, const xdcg_matrix *K, const xdcg_deflation *
                    T.nPUnits > 0 && T.nUnits <= kMaxGrid;
         };
         if (!build_units(R, kUnitRows, kProlongRows, false)) return XDCG_OOM;
+        if (!restrict_rows_prepare()) return XDCG_CUDA_ERROR;
         R.unitPart = dalloc<double>(c, 24 * (size_t)R.nUnits);
         R.boxTicket = dalloc<unsigned int>(c, S);
         if (!R.unitPart || !R.boxTicket) return XDCG_OOM;

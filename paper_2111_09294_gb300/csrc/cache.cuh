@@ -36,4 +36,16 @@ __device__ __forceinline__ float4 ld_keep(const float4 *a, uint64_t pol) {
     return v;
 }
 
+// asynchronous 4-byte copy into shared memory with the same policy; a thread
+// that reads back only what it copied itself needs no barrier, just the wait
+__device__ __forceinline__ void cp_keep(float *smem, const float *a, uint64_t pol) {
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 4, %2;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(smem)),
+                 "l"(a), "l"(pol)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_wait_all() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 }  // namespace xdcg

@@ -2,6 +2,8 @@
 // set-up, the FP64 inverse of E, and the per-iteration coarse solve
 // nu = E^-1 g that replaces the two solves of Algorithm 3 (their difference
 // lambda - mu = E^-1 (Z^T r - Z^T K y)) and the two of Algorithm 2.
+#include <type_traits>
+
 #include "cache.cuh"
 #include "reduce.cuh"
 
@@ -149,10 +151,11 @@ void launch_symmetrize(double *E, int k, cudaStream_t st) {
 // Scalar updates shared by the coarse kernels (modes as for k_coarse); blk
 // holds the block's share of nu^T (Z^T r) in thread 0 (the few row sums
 // gathered through shared memory: no FP64 shuffle tree in every warp).
+template <int THREADS>
 __device__ __forceinline__ void coarse_scalars(double blk, int mode, double *partials,
                                                Scalars *sc) {
     double tot[1];
-    if (grid_sum_t0(blk, partials, &sc->ticket[3], tot[0]) && threadIdx.x == 0) {
+    if (grid_sum_t0<THREADS>(blk, partials, &sc->ticket[3], tot[0]) && threadIdx.x == 0) {
         if (mode == 1) {
             sc->rho = sc->ry + tot[0];
             sc->beta = 0.0;
@@ -227,80 +230,125 @@ k_coarse(const double *__restrict__ Einv, int k, const double *__restrict__ g,
     double blk = 0.0;
     if (threadIdx.x == 0)
         for (int w = 0; w < kWarps; ++w) blk += rowPart[w];
-    coarse_scalars(blk, mode, partials, sc);
+    coarse_scalars<kThreads>(blk, mode, partials, sc);
 }
 
 // nu = E^-1 g with E^-1 held in FP32, for the FP32 iteration of the mixed
 // path.  A-DEF2 tolerates an inexact coarse solve (the coarse correction
 // acts as a preconditioner, not as a projection the recurrence relies on),
-// and on the test problems FP32 E^-1 changes no iteration count.  Two warps
-// per row, each streaming half of it with up to sixteen 16-byte loads in
-// flight per lane (rows are 16-byte aligned when k is a multiple of 4); g
-// comes as the FP32 copy the restriction writes, read through L1.  The two
-// halves are added in a fixed order.
+// and on the test problems FP32 E^-1 changes no iteration count.
+//
+// A block takes four rows, its two warps one half of the columns each, added
+// in that order; a lane keeps U loads per row in flight (16-byte ones when k
+// is a multiple of 4, so that rows are aligned), and an entry of g (the FP32
+// copy that the restriction writes, read through L1) serves the four rows.
+// E^-1 is set-up data: the first loads are issued before the wait for the
+// restriction.  Small blocks, because 810 of them (k = 3240) spread evenly
+// over the SMs and stay resident together.
+//
+// k = 3240 (42 MB of E^-1, from L2): 17.9 us before (a row per two warps, g read
+// for every row, few loads in flight), 15.9 now; k = 3150 (4-byte loads):
+// 16.0 before, 15.2 now; k = 60: 8.6 before,
+// 10.0 now.
+constexpr int kCoarse32Rows = 4, kCoarse32Threads = 64;
+
 template <int V>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kCoarse32Threads)
 k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
            const double *__restrict__ zr, double *nu, float *nu32, int mode, double *partials,
            Scalars *sc) {
-    pdl_wait();
-    if (sc->done != kRunning) return;
-    __shared__ float upper[kWarps / 2];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * (kWarps / 2) + (warp >> 1), h = warp & 1;
-    float s = 0.f;
-    if (i < k) {
-        const uint64_t keep = l2_keep_policy();
-        const float *row = Einv + (size_t)i * k;
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        if (V == 4) {
-            const int n4 = k >> 2, mid = (n4 + 1) >> 1;
-            const int j1 = h ? n4 : mid;
-            const float4 *r4 = reinterpret_cast<const float4 *>(row);
-            const float4 *g4 = reinterpret_cast<const float4 *>(g32);
-#pragma unroll 16
-            for (int j = (h ? mid : 0) + lane; j < j1; j += 32) {
-                const float4 a = ld_keep(r4 + j, keep), x = __ldg(g4 + j);
-                s0 = fmaf(a.x, x.x, s0);
-                s1 = fmaf(a.y, x.y, s1);
-                s2 = fmaf(a.z, x.z, s2);
-                s3 = fmaf(a.w, x.w, s3);
-            }
-        } else {
-            const int mid = (k + 1) >> 1, j1 = h ? k : mid;
-#pragma unroll 16
-            for (int j = (h ? mid : 0) + lane; j < j1; j += 32)
-                s0 = fmaf(ld_keep(row + j, keep), __ldg(g32 + j), s0);
-        }
-        s = (s0 + s1) + (s2 + s3);
+    constexpr int R = kCoarse32Rows, U = V == 4 ? 4 : 8;
+    using E = typename std::conditional<V == 4, float4, float>::type;
+    __shared__ float upper[R];
+    const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i0 = blockIdx.x * R;
+    const int nv = k / V, mid = (nv + 1) >> 1;
+    const int j0 = (h ? mid : 0) + lane, j1 = h ? nv : mid;
+    const uint64_t keep = l2_keep_policy();
+    const E *row[R];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    }
-    if (lane == 0 && h == 1) upper[warp >> 1] = s;
-    __syncthreads();
-    __shared__ double rowPart[kWarps / 2];
-    if (lane == 0 && h == 0) {
-        double part = 0.0;
-        if (i < k) {
-            const float v = s + upper[warp >> 1];
-            nu[i] = (double)v;
-            nu32[i] = v;
-            if (mode != 0) part = (double)v * zr[i];
+    for (int r = 0; r < R; ++r)
+        row[r] = reinterpret_cast<const E *>(Einv + (size_t)min(i0 + r, k - 1) * k);
+    E e[U][R];
+    auto load = [&](int j) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j + 32 * u < j1)
+#pragma unroll
+                for (int r = 0; r < R; ++r) e[u][r] = ld_keep(row[r] + j + 32 * u, keep);
+    };
+    // a launch queued past a stop loads nothing; this early read of the flag
+    // may be stale, the one after the wait decides
+    const bool early = __ldcg(&sc->done) == kRunning;
+    if (early) load(j0);
+    pdl_wait();
+    pdl_trigger();
+    if (sc->done != kRunning) return;
+    if (!early) load(j0);
+    float s[R][4] = {};
+    const E *gv = reinterpret_cast<const E *>(g32);
+    for (int j = j0; j < j1; j += 32 * U) {
+        E x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j + 32 * u < j1) x[u] = __ldg(gv + j + 32 * u);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (j + 32 * u < j1) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if constexpr (V == 4) {
+                        s[r][0] = fmaf(e[u][r].x, x[u].x, s[r][0]);
+                        s[r][1] = fmaf(e[u][r].y, x[u].y, s[r][1]);
+                        s[r][2] = fmaf(e[u][r].z, x[u].z, s[r][2]);
+                        s[r][3] = fmaf(e[u][r].w, x[u].w, s[r][3]);
+                    } else {
+                        s[r][0] = fmaf(e[u][r], x[u], s[r][0]);
+                    }
+                }
+            }
         }
-        rowPart[warp >> 1] = part;
+        load(j + 32 * U);
     }
+    // the rows' sums over the lanes by halving exchanges: lane 8 r gets row r
+    float v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = (s[r][0] + s[r][1]) + (s[r][2] + s[r][3]);
+#pragma unroll
+    for (int half = 2, o = 16; half > 0; half >>= 1, o >>= 1) {
+        const bool hi = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const float send = hi ? v[i] : v[i + half], mine = hi ? v[i + half] : v[i];
+            v[i] = mine + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    const int r = lane >> 3, i = i0 + r;
+    const bool holder = (lane & 7) == 0;
+    if (h == 1 && holder) upper[r] = v[0];
     __syncthreads();
     double blk = 0.0;
-    if (threadIdx.x == 0)
-        for (int r = 0; r < kWarps / 2; ++r) blk += rowPart[r];
-    coarse_scalars(blk, mode, partials, sc);
+    if (h == 0) {
+        double part = 0.0;
+        if (holder && i < k) {
+            const float t = v[0] + upper[r];
+            nu[i] = (double)t;
+            nu32[i] = t;
+            if (mode != 0) part = (double)t * zr[i];
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q) blk += __shfl_sync(0xffffffffu, part, 8 * q);
+    }
+    coarse_scalars<kCoarse32Threads>(blk, mode, partials, sc);
 }
 
 void launch_coarse32(const float *Einv, int k, const float *g32, const double *zr, double *nu,
                      float *nu32, int mode, double *partials, Scalars *sc, cudaStream_t st) {
-    const int grid = (k + kWarps / 2 - 1) / (kWarps / 2);
-    launch_pdl(k % 4 == 0 ? k_coarse32<4> : k_coarse32<1>, grid > 0 ? grid : 1, kThreads, 0, st,
-               Einv, k, g32, zr, nu, nu32, mode, partials, sc);
+    const int grid = (k + kCoarse32Rows - 1) / kCoarse32Rows;
+    launch_pdl(k % 4 == 0 ? k_coarse32<4> : k_coarse32<1>, grid > 0 ? grid : 1, kCoarse32Threads,
+               0, st, Einv, k, g32, zr, nu, nu32, mode, partials, sc);
 }
 
 void launch_coarse(const double *Einv, int k, const double *g, const double *zr, double *nu,

@@ -244,6 +244,7 @@ void launch_restrict_update(const RowBoxDev &B, float *u, const float *r_cur, fl
                             const float *p, const float *q, int mode, double *g, double *zr,
                             double *partials, Scalars *sc, cudaStream_t st,
                             const float *y = nullptr);
+bool restrict_rows_prepare();
 void launch_prolong_rows(const RowBoxDev &B, const float *nu32, const float *y, float *p,
                          int mode, Scalars *sc, cudaStream_t st);
 // The FP32 iteration's restriction (mode 0) after a product launched with

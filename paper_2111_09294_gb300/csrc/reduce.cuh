@@ -37,8 +37,52 @@ __device__ __forceinline__ void block_sum(A (&v)[NV]) {
     if (w == 0) {
 #pragma unroll
         for (int i = 0; i < NV; ++i) v[i] = (l < nw) ? sm[i][l] : A(0);
-        warp_sum<A, NV>(v);
+        // eight warps or fewer: the tree's first two levels would add zeros
+        if (nw <= 8) {
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+                for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+        } else {
+            warp_sum<A, NV>(v);
+        }
     }
+}
+
+// Sums N <= P values over the warp by halving exchanges, P - 1 shuffles (and,
+// for P = 16, one more) instead of 5 N: each value's tree is that of warp_sum
+// (pairs 16, 8, 4, 2, 1 lanes apart).  Lane l gets the total of value l (P =
+// 32) or l >> 1 (P = 16).
+template <int P, int N>
+__device__ __forceinline__ float warp_sum_scatter(const float (&in)[N]) {
+    static_assert((P == 16 || P == 32) && N <= P, "");
+    float v[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) v[i] = i < N ? in[i < N ? i : 0] : 0.0f;
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int half = P / 2; half > 0; half >>= 1) {
+        const bool hi = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const float send = hi ? v[i] : v[i + half];
+            const float keep = hi ? v[i + half] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        o >>= 1;
+    }
+    if (P == 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return v[0];
+}
+
+// The second stage of block_sum for eight warps' sums of one value (the tree
+// over 32 lanes of which eight hold a value: zeros added twice, then 4, 2, 1).
+__device__ __forceinline__ float sum_of_8(const float (&x)[8]) {
+    float y[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) y[w] = x[w] + 0.0f;
+    return ((y[0] + y[4]) + (y[2] + y[6])) + ((y[1] + y[5]) + (y[3] + y[7]));
 }
 
 // The last block's share of a grid-wide sum: value i of the nblk blocks'
@@ -137,42 +181,37 @@ __device__ __forceinline__ float2 df_of(double v) {
 }
 
 // The total of n block partials (double-float) a previous kernel stored
-// (kFinDefer and the FP32 iteration's deferred sums): every thread loads its
-// share at once (one round trip), the shares are added in a fixed order
-// within each thread, by a tree over the lanes and over the warps, so every
-// block of the consuming kernel gets the same bits; valid in every thread.
-// Replaces the producer's ticketed last-block reduction (fence, atomic, the
-// last block's tail).
-__device__ __forceinline__ double block_read_total(const float2 *partials, int n) {
-    constexpr int kLoads = 8;
+// (kFinDefer): every thread loads its share at once (one round trip), the
+// shares are added in a fixed order within each thread, by a tree over the
+// lanes and over the warps, so every block of the consuming kernel gets the
+// same bits.  Valid in thread 0 (FP64 instructions cost 64 cycles each
+// whatever the number of threads, and all of a block's warps would share the
+// SM's FP64 units: one thread goes on alone).  A share that is not there is
+// not added: a normalised pair plus zero is itself.
+__device__ __forceinline__ double block_total_t0(const float2 *partials, int n) {
     __shared__ float2 wsum[32];
-    __shared__ double total;
     const int t = threadIdx.x, nt = blockDim.x;
-    float2 v[kLoads];
-#pragma unroll
-    for (int q = 0; q < kLoads; ++q) {
-        const int i = t + q * nt;
-        v[q] = i < n ? __ldcg(partials + i) : make_float2(0.f, 0.f);
-    }
-    float2 acc = v[0];
-#pragma unroll
-    for (int q = 1; q < kLoads; ++q) acc = df_add(acc, v[q]);
-    for (int i = t + kLoads * nt; i < n; i += nt) acc = df_add(acc, __ldcg(partials + i));
+    const float2 none = make_float2(0.f, 0.f);
+    float2 a = t < n ? __ldcg(partials + t) : none;
+    float2 b = t + nt < n ? __ldcg(partials + t + nt) : none;
+    if (nt < n) a = df_add(a, b);
+    for (int i = t + 2 * nt; i - t < n; i += nt)
+        a = df_add(a, i < n ? __ldcg(partials + i) : none);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         float2 other;
-        other.x = __shfl_xor_sync(0xffffffffu, acc.x, o);
-        other.y = __shfl_xor_sync(0xffffffffu, acc.y, o);
-        acc = df_add(acc, other);
+        other.x = __shfl_xor_sync(0xffffffffu, a.x, o);
+        other.y = __shfl_xor_sync(0xffffffffu, a.y, o);
+        a = df_add(a, other);
     }
-    if ((t & 31) == 0) wsum[t >> 5] = acc;
+    if ((t & 31) == 0) wsum[t >> 5] = a;
     __syncthreads();
+    double total = 0.0;
     if (t == 0) {
         float2 s = wsum[0];
         for (int w = 1; w < (nt >> 5); ++w) s = df_add(s, wsum[w]);
         total = (double)s.x + (double)s.y;
     }
-    __syncthreads();
     return total;
 }
 
@@ -183,12 +222,19 @@ __device__ __forceinline__ bool grid_sum(A (&v)[NV], double *partials, unsigned 
     return grid_sum_of<A, NV>(v, partials, ticket, tot, (int)blockIdx.x, (int)gridDim.x);
 }
 
-// Grid-wide sum of one value already reduced to thread 0 of each block:
-// returns true in the last block to finish, where thread 0 holds the FP64
-// total (block partials added in block order).
+// Grid-wide sum of one value already reduced to thread 0 of each block of
+// THREADS threads: returns true in the last block to finish, where thread 0
+// holds the FP64 total.  The order of the sum is that of 256 threads whatever
+// THREADS: slot t = 0 .. 255 adds partials t, t + 256, ..., then the tree over
+// the 32 slots of a warp and the tree over the eight warps; a thread of a
+// smaller block takes 256 / THREADS slots.
+template <int THREADS>
 __device__ __forceinline__ bool grid_sum_t0(double v, double *partials, unsigned int *ticket,
                                             double &tot) {
+    constexpr int Q = kThreads / THREADS;
+    static_assert(Q == 1 || Q == 4, "");
     __shared__ bool last;
+    __shared__ double sums[kWarps];
     if (threadIdx.x == 0) {
         partials[blockIdx.x] = v;
         __threadfence();
@@ -197,12 +243,38 @@ __device__ __forceinline__ bool grid_sum_t0(double v, double *partials, unsigned
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    double s[1] = {0.0};
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s[0] += __ldcg(partials + b);
-    block_sum<double, 1>(s);
-    if (threadIdx.x == 0) {
-        tot = s[0];
-        *ticket = 0u;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = (int)gridDim.x;
+    double s[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) s[q] = 0.0;
+    for (int b = threadIdx.x; b < n; b += kThreads)
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (b + q * THREADS < n) s[q] += __ldcg(partials + b + q * THREADS);
+    int o = 16;
+    if (Q == 4) {   // halving exchanges: lanes 8 q .. 8 q + 7 keep the sums of slot set q
+#pragma unroll
+        for (int half = 2; half > 0; half >>= 1, o >>= 1) {
+            const bool hi = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < half; ++i) {
+                const double send = hi ? s[i] : s[(i + half) % Q];
+                const double mine = hi ? s[(i + half) % Q] : s[i];
+                s[i] = mine + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+    }
+    for (; o > 0; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+    if (lane % (32 / Q) == 0) sums[warp + (THREADS / 32) * (lane / (32 / Q))] = s[0];
+    __syncthreads();
+    if (warp == 0) {
+        double t = lane < kWarps ? sums[lane] : 0.0;
+#pragma unroll
+        for (int p = 4; p > 0; p >>= 1) t += __shfl_xor_sync(0xffffffffu, t, p);
+        if (lane == 0) {
+            tot = t;
+            *ticket = 0u;
+        }
     }
     return true;
 }

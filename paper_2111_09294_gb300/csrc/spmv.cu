@@ -255,7 +255,7 @@ k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__rest
         __syncwarp();
     }
     if (fin == kFinDefer) {
-        // the next kernel adds the blocks' sums (block_read_total); a failed
+        // the next kernel adds the blocks' sums (block_total_t0); a failed
         // wait is in sc->fault, which it reads too
         block_sum<T, 1>(part);
         if (threadIdx.x == 0)
@@ -375,6 +375,7 @@ k_spmv_lean(SpmvDev<float> A, const float *__restrict__ x, float *__restrict__ y
     if (early)
         while (pmore && issued < NS) issue();
     pdl_wait();
+    pdl_trigger();
     if (sc->done != kRunning) {
         const unsigned long long drain = global_ns() + kDrainNs;
         for (int k = 0; k < issued; ++k) mbar_wait(bars + k % NS, (uint32_t)(k / NS) & 1u, drain);

@@ -39,3 +39,19 @@ def test_precond_box_sizes(m, n_box, form):
     ref = O.adef2_apply(K, M, Co, r)
     assert np.linalg.norm(z - ref) <= 1e-8 * np.linalg.norm(ref)
     s.close()
+
+
+# the FP32 iteration's row kernels: one unit per SM and many units (216 boxes),
+# rows beyond the ones in flight before the wait (9, 1), coarse dimensions that
+# are multiples of 4 and not.  tol 1e-12 and u to 1e-7 as for every mixed solve.
+@pytest.mark.parametrize("m,n_box", SIZES + [(13, 6)])
+def test_mixed_box_sizes(m, n_box):
+    from paper_2111_09294_gb300 import Solver
+    P = X.build_problem(m, [C.PlanarEdgeCrack(0.5, 0.41, 1.25 / m)], n_box)
+    K, M, Co = O.setup(P)
+    ref = O.adef2_pcg(K, P.f, M, Co, tol=1e-12)
+    s = Solver.from_problem(P, precision="mixed")
+    u, info = s.solve(torch.tensor(P.f, device="cuda"), tol=1e-12)
+    assert info["rel_res_true"] <= 1e-12
+    assert np.linalg.norm(u.cpu().numpy() - ref.u) <= 1e-7 * np.linalg.norm(ref.u)
+    s.close()

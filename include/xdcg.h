@@ -171,7 +171,7 @@ typedef struct {
                                 Default 0: the default shape (FP32 5, FP64 0).  Two contexts
                                 with different shapes may round the fused dot differently */
     int32_t graph;           /* 1: the loops of the solves enqueue their iterations as CUDA
-                                graphs: a batch of 8 iterations of xdcg_solve / xdcg_solve_x0
+                                graphs: a batch of 4 iterations of xdcg_solve / xdcg_solve_x0
                                 (FP64, and MIXED's FP32 iteration) is recorded by stream capture
                                 once per context (on a private stream of the context, so the
                                 context's own stream may be the legacy default stream) and

@@ -22,7 +22,10 @@ using namespace xdcg;
 
 namespace {
 
-constexpr int kBatch = 8;              // iterations enqueued between convergence polls
+constexpr int kStallEvery = 8;         // iterations between stall tests
+constexpr int kUnitIts = 4;            // iterations enqueued (or recorded in a graph) together
+static_assert(kStallEvery % kUnitIts == 0, "");
+constexpr int kAheadIts = 2;           // enqueued when this many are left past the last report
 constexpr int kMaxGrid = 1 << 16;      // partial-sum slots per reduction value
 
 struct Level64 {
@@ -103,8 +106,7 @@ struct xdcg_ctx {
     double *partials = nullptr;
     Scalars *sc = nullptr, *sc32 = nullptr, *aux = nullptr;
     Scalars *h_sc = nullptr;   // pinned
-    int *h_done = nullptr;     // pinned, 2 slots
-    Scalars *h_poll = nullptr; // pinned, 2 slots: the FP32 run's scalars at each poll
+    Progress *h_prog = nullptr; // pinned: what the running solve reports per iteration
     cudaEvent_t ev0 = nullptr, ev1 = nullptr, evb[2] = {nullptr, nullptr};
     std::vector<cudaEvent_t> evS, evE;
     std::vector<cudaEvent_t> evP;      // per-kernel marks of timed iterations (time_spmv = 2)
@@ -261,20 +263,21 @@ bool points_collinear(const std::vector<double> &x) {
 }
 
 __global__ void k_init_scalars(Scalars *sc, double tol2, const double *ffsrc, int max_it,
-                               double *hist, int histCap) {
+                               Progress *prog, double *hist, int histCap) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         Scalars z{};
         z.tol2ff = ffsrc ? tol2 * (*ffsrc) : tol2;
         z.max_it = max_it;
         z.hist = hist;
         z.histCap = histCap;
+        z.prog = prog;
         *sc = z;
     }
 }
 
 void init_scalars(xdcg_ctx *c, Scalars *sc, double tol2, const double *ffsrc, int max_it,
-                  double *hist = nullptr, int histCap = 0) {
-    k_init_scalars<<<1, 32, 0, c->st>>>(sc, tol2, ffsrc, max_it, hist, histCap);
+                  Progress *prog = nullptr, double *hist = nullptr, int histCap = 0) {
+    k_init_scalars<<<1, 32, 0, c->st>>>(sc, tol2, ffsrc, max_it, prog, hist, histCap);
     c->launches++;
 }
 
@@ -324,6 +327,62 @@ xdcg_status phase_collect(xdcg_ctx *c, int n, int P, xdcg_result *res) {
         }                                                                       \
     } while (0)
 
+// Follows a run by its reports (Progress).  The host enqueues the next kUnitIts
+// iterations when kAheadIts are left past the last one reported: the device
+// never waits for it, at most kAheadIts + kUnitIts - 1 iterations are queued
+// past a stop (four or five launches of ~2 us each; 8 to 16 with a stream copy
+// and an event per 8 iterations before), and nothing is read back through the
+// stream.  Per FP32 iteration 12^3 31.8 -> 27.2 us, 48^3 84.7 -> 78.0 us.
+struct RunFollower {
+    xdcg_ctx *c;
+    int seen;                     // the last iteration reported
+    bool stopped = false, lost = false;   // lost: the device went idle without a report
+    double rr = 0.0;              // ||r||^2 of iteration seen
+    RunFollower(xdcg_ctx *ctx, int it0) : c(ctx), seen(it0 - 1) {}
+    // forget what the slot of iteration it held (before its launch)
+    static void clear(xdcg_ctx *c, int it) {
+        __atomic_store_n(&c->h_prog->rr[it % kRing], kNoReport, __ATOMIC_RELAXED);
+    }
+    bool take(int it) {
+        const unsigned long long v = __atomic_load_n(&c->h_prog->rr[it % kRing], __ATOMIC_ACQUIRE);
+        if (v == kNoReport) return false;
+        stopped = (v >> 63) != 0;
+        const unsigned long long a = v & 0x7fffffffffffffffull;
+        std::memcpy(&rr, &a, sizeof(rr));
+        seen = it;
+        return true;
+    }
+    // waits for iteration it = seen + 1, which has been launched
+    void next() {
+        const int it = seen + 1;
+        for (unsigned int spin = 1; !take(it); ++spin) {
+            // a stop at an earlier iteration (a failed wait) is reported in
+            // that iteration's slot; a device error ends in an idle stream
+            if (spin % 1024 == 0 && cudaStreamQuery(c->st) != cudaErrorNotReady) {
+                if (take(it)) return;
+                lost = true;
+                return;
+            }
+        }
+    }
+    // the run's iterations and done flag, once stopped (or the device is idle)
+    xdcg_status finish(const Scalars *sc, int *its_out, int *done_out) {
+        if (stopped) {
+            const unsigned long long s = __atomic_load_n(&c->h_prog->stop, __ATOMIC_ACQUIRE);
+            *its_out = (int)(s >> 32);
+            *done_out = (int)(s & 0xffffffffull);
+        } else {
+            CK(cudaMemcpyAsync(c->h_sc, sc, sizeof(Scalars), cudaMemcpyDeviceToHost, c->st));
+            CK(cudaStreamSynchronize(c->st));
+            *its_out = c->h_sc->its;
+            *done_out = c->h_sc->done;
+            rr = c->h_sc->rr;
+        }
+        CK(cudaGetLastError());
+        return XDCG_OK;
+    }
+};
+
 // ---- one preconditioned CG run (Algorithms 1-3) ----------------------------
 
 // Unscaled path: block-Jacobi applied by the node-block factors, Z from
@@ -360,7 +419,7 @@ struct PlainPath {
 template <typename T, typename Path>
 xdcg_status run_pcg(xdcg_ctx *c, Path path, const T *f, T *u, T *r, T *p, T *q, T *y,
                     Scalars *sc, int max_it, bool guess, int *its_out, int *done_out,
-                    xdcg_result *res) {
+                    double *rr_out, xdcg_result *res) {
     cudaStream_t st = c->st;
     const bool timeSpmv = c->opt.time_spmv == 1, timeKernels = c->opt.time_spmv == 2;
     if (guess) {
@@ -386,7 +445,7 @@ xdcg_status run_pcg(xdcg_ctx *c, Path path, const T *f, T *u, T *r, T *p, T *q, 
     c->launches += 5;
 
     int launched = 0;
-    const int max_batches = max_it / kBatch + 2;
+    const int limit = (max_it / kStallEvery + 2) * kStallEvery;
     // opt.graph: the batch's kernels as one recorded graph (not with the
     // timing modes, whose events sit between the kernels)
     const bool useGraph = c->opt.graph && !timeSpmv && !timeKernels;
@@ -395,7 +454,7 @@ xdcg_status run_pcg(xdcg_ctx *c, Path path, const T *f, T *u, T *r, T *p, T *q, 
         xdcg_status s = loop_graph(c, c->loop64, key, [&](cudaStream_t cs) {
             Path rec = path;
             rec.st = cs;
-            for (int i = 0; i < kBatch; ++i) {
+            for (int i = 0; i < kUnitIts; ++i) {
                 rec.spmv(p, q, nullptr, 0, kFinAlpha, sc);
                 rec.update(u, r, p, q, y, 0, sc);
                 rec.restrict_(r, y, 1, c->zr, sc);
@@ -406,52 +465,56 @@ xdcg_status run_pcg(xdcg_ctx *c, Path path, const T *f, T *u, T *r, T *p, T *q, 
         });
         if (s != XDCG_OK) return s;
     }
-    for (int b = 0; b < max_batches; ++b) {
-        if (useGraph) {
-            CK(cudaGraphLaunch(c->loop64.exec, st));
-            c->launches += c->loop64.launches;
-            c->graphLaunches++;
-            launched += kBatch;
-        }
-        for (int i = 0; i < kBatch && !useGraph; ++i) {
-            if (timeSpmv) {
-                if ((int)c->evS.size() <= launched) {
-                    cudaEvent_t e0, e1;
-                    CK(cudaEventCreate(&e0));
-                    CK(cudaEventCreate(&e1));
-                    c->evS.push_back(e0);
-                    c->evE.push_back(e1);
-                }
-                CK(cudaEventRecord(c->evS[launched], st));
+    RunFollower run(c, 0);
+    while (!run.stopped && !run.lost) {
+        if (launched < limit && launched - run.seen <= kAheadIts) {
+            for (int i = 1; i <= kUnitIts; ++i) RunFollower::clear(c, launched + i);
+            if (useGraph) {
+                CK(cudaGraphLaunch(c->loop64.exec, st));
+                c->launches += c->loop64.launches;
+                c->graphLaunches++;
+                launched += kUnitIts;
+                continue;
             }
-            MARK(launched, 0);
-            path.spmv(p, q, nullptr, 0, kFinAlpha, sc);
-            if (timeSpmv) CK(cudaEventRecord(c->evE[launched], st));
-            MARK(launched, 1);
-            path.update(u, r, p, q, y, 0, sc);
-            MARK(launched, 2);
-            path.restrict_(r, y, 1, c->zr, sc);
-            MARK(launched, 3);
-            path.coarse(c->zr, 2, sc);
-            MARK(launched, 4);
-            path.prolong(y, p, 0, sc);
-            MARK(launched, 5);
-            c->launches += 5;
-            ++launched;
-        }
-        CK(cudaMemcpyAsync(&c->h_done[b & 1], &sc->done, sizeof(int), cudaMemcpyDeviceToHost, st));
-        CK(cudaEventRecord(c->evb[b & 1], st));
-        if (b >= 1) {
-            CK(cudaEventSynchronize(c->evb[(b - 1) & 1]));
-            if (c->h_done[(b - 1) & 1] != kRunning) break;
+            for (int i = 0; i < kUnitIts; ++i) {
+                if (timeSpmv) {
+                    if ((int)c->evS.size() <= launched) {
+                        cudaEvent_t e0, e1;
+                        CK(cudaEventCreate(&e0));
+                        CK(cudaEventCreate(&e1));
+                        c->evS.push_back(e0);
+                        c->evE.push_back(e1);
+                    }
+                    CK(cudaEventRecord(c->evS[launched], st));
+                }
+                MARK(launched, 0);
+                path.spmv(p, q, nullptr, 0, kFinAlpha, sc);
+                if (timeSpmv) CK(cudaEventRecord(c->evE[launched], st));
+                MARK(launched, 1);
+                path.update(u, r, p, q, y, 0, sc);
+                MARK(launched, 2);
+                path.restrict_(r, y, 1, c->zr, sc);
+                MARK(launched, 3);
+                path.coarse(c->zr, 2, sc);
+                MARK(launched, 4);
+                path.prolong(y, p, 0, sc);
+                MARK(launched, 5);
+                c->launches += 5;
+                ++launched;
+            }
+        } else if (run.seen < launched) {
+            run.next();
+        } else {
+            break;
         }
     }
-    CK(cudaMemcpyAsync(c->h_sc, sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    CK(cudaGetLastError());
-    *its_out = c->h_sc->its;
-    *done_out = c->h_sc->done;
-    const int nt = std::min(launched, c->h_sc->its);
+    {
+        xdcg_status s = run.finish(sc, its_out, done_out);
+        if (s != XDCG_OK) return s;
+    }
+    *rr_out = run.rr;
+    const int nt = std::min(launched, *its_out);
+    if (timeSpmv || timeKernels) CK(cudaStreamSynchronize(st));
     if (timeSpmv) {
         for (int i = 0; i < nt; ++i) {
             float ms = 0.f;
@@ -476,14 +539,20 @@ xdcg_status run_pcg(xdcg_ctx *c, Path path, const T *f, T *u, T *r, T *p, T *q, 
 // writes the new one of its own.  Iteration i reads residual buffer
 // (i & 1 ? rB : rA) and writes the other.
 
-__global__ void k_set_trigger(Scalars *sc, int mode, double delta2, double floor2) {
+__global__ void k_set_trigger(Scalars *sc, int mode, double delta2, double target2,
+                              double true2) {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         if (mode == 0) {            // re-arm without a convergence test; keep the
             sc->done = kRunning;    // recursive ||r||^2 for the restart test
             sc->tol2ff = -1.0;
             sc->scratch[3] = sc->rr;
-        } else {                    // next residual replacement when ||r||^2 drops below this
-            sc->tol2ff = fmax(delta2 * sc->rr, floor2);
+        } else {
+            // next residual replacement when ||r||^2 drops by delta2, or to
+            // target2 scaled by ||r||^2 / true2, but by a factor 100 first
+            // (target2 = 0: by delta2)
+            const double gamma2 = sc->rr / true2;
+            const double a = target2 * gamma2, b = kMinGroupDrop2 * sc->rr;
+            sc->tol2ff = fmax(delta2 * sc->rr, b < a ? b : a);
         }
     }
 }
@@ -530,21 +599,20 @@ void scaled_init(xdcg_ctx *c, const float *f, float *u, float *rA, float *p, Sca
 // rounding of K~ hides the components still to be resolved.
 constexpr int kStallIts = 200;
 
-// Run iterations (in batches, polling the device flag) until a kernel stops
-// the run (the replacement trigger, breakdown, the iteration cap) or the run
-// stalls (*stalled, the device flag still running).
+// Run iterations from iteration it0 on, following the device's reports, until a
+// kernel stops the run (the replacement trigger, breakdown, the iteration cap)
+// or the run stalls (*stalled, the device flag still running).  The stall test
+// looks at every kStallEvery-th iteration; a stall found there ends the run
+// kStallEvery iterations later.
 xdcg_status scaled_iterate(xdcg_ctx *c, float *u, float *rA, float *rB, float *p, float *q,
-                           Scalars *sc, int max_it, int *its_out, int *done_out,
-                           xdcg_result *res, bool *stalled) {
+                           Scalars *sc, int max_it, int it0, int *its_out, int *done_out,
+                           double *rr_out, xdcg_result *res, bool *stalled) {
     cudaStream_t st = c->st;
     Level32 &L = c->L32;
     const bool timeSpmv = c->opt.time_spmv == 1, timeKernels = c->opt.time_spmv == 2;
-    CK(cudaMemcpyAsync(c->h_sc, sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    const int it0 = c->h_sc->its;
     int i = it0, launched = 0;
-    const int max_batches = (max_it - it0) / kBatch + 2;
-    double bestRR = c->h_sc->rr;
+    const int limit = ((max_it - it0) / kStallEvery + 2) * kStallEvery;
+    double bestRR = 0.0;
     int lastGain = it0;
     *stalled = false;
     // kernel m (0..3) of iteration it of the FP32 iteration, enqueued on s
@@ -581,72 +649,80 @@ xdcg_status scaled_iterate(xdcg_ctx *c, float *u, float *rA, float *rB, float *p
         }
     };
     // opt.graph: a batch's kernels as one recorded graph per residual-buffer
-    // parity of its first iteration (kBatch is even), not with the timing
+    // parity of its first iteration (kUnitIts is even), not with the timing
     // modes, whose events sit between the kernels
     const bool useGraph = c->opt.graph && !timeSpmv && !timeKernels;
     LoopGraph &G = c->loop32[it0 & 1];
     if (useGraph) {
         const LoopKey key{u, rA, rB, p, q, sc, c->zr, c->userBlocks ? c->y32 : nullptr};
         xdcg_status s = loop_graph(c, G, key, [&](cudaStream_t cs) {
-            for (int j = 0; j < kBatch; ++j)
+            for (int j = 0; j < kUnitIts; ++j)
                 for (int m = 0; m < 4; ++m) kernel(m, it0 + j, cs);
         });
         if (s != XDCG_OK) return s;
     }
-    for (int b = 0; b < max_batches; ++b) {
-        if (useGraph) {
-            CK(cudaGraphLaunch(G.exec, st));
-            c->launches += G.launches;
-            c->graphLaunches++;
-            i += kBatch;
-            launched += kBatch;
-        }
-        for (int j = 0; j < kBatch && !useGraph; ++j, ++i, ++launched) {
-            if (timeSpmv) {
-                if ((int)c->evS.size() <= launched) {
-                    cudaEvent_t e0, e1;
-                    CK(cudaEventCreate(&e0));
-                    CK(cudaEventCreate(&e1));
-                    c->evS.push_back(e0);
-                    c->evE.push_back(e1);
+    RunFollower run(c, it0);
+    int stopAt = limit;           // iterations to launch at most
+    while (!run.stopped && !run.lost) {
+        if (launched < stopAt && launched - (run.seen - it0) <= kAheadIts) {
+            for (int j = 1; j <= kUnitIts; ++j) RunFollower::clear(c, i + j);
+            if (useGraph) {
+                CK(cudaGraphLaunch(G.exec, st));
+                c->launches += G.launches;
+                c->graphLaunches++;
+                i += kUnitIts;
+                launched += kUnitIts;
+                continue;
+            }
+            for (int j = 0; j < kUnitIts; ++j, ++i, ++launched) {
+                if (timeSpmv) {
+                    if ((int)c->evS.size() <= launched) {
+                        cudaEvent_t e0, e1;
+                        CK(cudaEventCreate(&e0));
+                        CK(cudaEventCreate(&e1));
+                        c->evS.push_back(e0);
+                        c->evE.push_back(e1);
+                    }
+                    CK(cudaEventRecord(c->evS[launched], st));
                 }
-                CK(cudaEventRecord(c->evS[launched], st));
+                MARK(launched, 0);
+                kernel(0, i, st);
+                if (timeSpmv) CK(cudaEventRecord(c->evE[launched], st));
+                MARK(launched, 1);
+                kernel(1, i, st);
+                MARK(launched, 2);
+                kernel(2, i, st);
+                MARK(launched, 3);
+                kernel(3, i, st);
+                MARK(launched, 4);
             }
-            MARK(launched, 0);
-            kernel(0, i, st);
-            if (timeSpmv) CK(cudaEventRecord(c->evE[launched], st));
-            MARK(launched, 1);
-            kernel(1, i, st);
-            MARK(launched, 2);
-            kernel(2, i, st);
-            MARK(launched, 3);
-            kernel(3, i, st);
-            MARK(launched, 4);
-        }
-        // one copy per poll: the stop flag and ||r||^2 for the stall test
-        CK(cudaMemcpyAsync(&c->h_poll[b & 1], sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
-        CK(cudaEventRecord(c->evb[b & 1], st));
-        if (b >= 1) {
-            CK(cudaEventSynchronize(c->evb[(b - 1) & 1]));
-            if (c->h_poll[(b - 1) & 1].done != kRunning) break;
-            const double rrNow = c->h_poll[(b - 1) & 1].rr;
-            const int itNow = it0 + b * kBatch;
-            if (rrNow < 0.81 * bestRR) {
-                bestRR = rrNow;
-                lastGain = itNow;
-            } else if (itNow - lastGain >= kStallIts) {
-                *stalled = true;
-                break;
+        } else if (run.seen < it0 + launched) {
+            run.next();
+            if (run.stopped || run.lost) break;
+            const int ran = run.seen - it0;
+            if (ran == 0) {
+                bestRR = run.rr;   // the residual the run starts from
+            } else if (ran % kStallEvery == 0) {
+                if (run.rr < 0.81 * bestRR) {
+                    bestRR = run.rr;
+                    lastGain = run.seen;
+                } else if (run.seen - lastGain >= kStallIts && !*stalled) {
+                    *stalled = true;
+                    stopAt = ran + kStallEvery;
+                }
             }
+        } else {
+            break;
         }
     }
-    CK(cudaMemcpyAsync(c->h_sc, sc, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    CK(cudaGetLastError());
-    *its_out = c->h_sc->its;
-    *done_out = c->h_sc->done;
+    {
+        xdcg_status s = run.finish(sc, its_out, done_out);
+        if (s != XDCG_OK) return s;
+    }
+    *rr_out = run.rr;
     if (*done_out != kRunning) *stalled = false;
-    const int nt = std::min(launched, c->h_sc->its - it0);
+    const int nt = std::min(launched, *its_out - it0);
+    if (timeSpmv || timeKernels) CK(cudaStreamSynchronize(st));
     if (timeSpmv) {
         for (int e = 0; e < nt; ++e) {
             float ms = 0.f;
@@ -678,14 +754,15 @@ xdcg_status solve_fp64(xdcg_ctx *c, const double *f, double *u, double tol, bool
     cudaStream_t st = c->st;
     init_scalars(c, c->aux, -1.0, nullptr, INT_MAX);
     launch_dot<double>(f, f, c->n, c->partials, c->aux, kFinStore, 0, st);
-    init_scalars(c, c->sc, tol * tol, &c->aux->scratch[0], c->opt.max_iter, c->hist,
+    init_scalars(c, c->sc, tol * tol, &c->aux->scratch[0], c->opt.max_iter, c->h_prog, c->hist,
                  c->hist ? c->opt.max_iter + 1 : 0);
     c->launches += 1;
     int its = 0, done = 0;
+    double rr = 0.0;
+    RunFollower::clear(c, 0);
     xdcg_status s = run_pcg<double>(c, PlainPath{c, c->L64, c->st}, f, u, c->r64, c->p64, c->q64,
-                                    c->y64, c->sc, c->opt.max_iter, guess, &its, &done, res);
+                                    c->y64, c->sc, c->opt.max_iter, guess, &its, &done, &rr, res);
     if (s != XDCG_OK) return s;
-    const double rr = c->h_sc->rr;
     // true residual f - K u in FP64
     launch_spmv<double>(c->L64.A, u, c->r64, f, 1, c->partials, c->aux, kFinStore, 1, st);
     c->launches += 1;
@@ -748,20 +825,22 @@ xdcg_status solve_mixed(xdcg_ctx *c, const double *f, double *u, double tol, boo
     launch_fwd_scale(c->nNodes, L.dofStart64, L.dofStart64, L.dofStart32, L.F, rhs, s0, c->f32,
                      st);
     CK(cudaMemsetAsync(c->u32, 0, c->n * sizeof(float), st));
-    init_scalars(c, c->sc32, -1.0, nullptr, c->opt.max_iter);
+    init_scalars(c, c->sc32, -1.0, nullptr, c->opt.max_iter, c->h_prog);
+    RunFollower::clear(c, 0);
     scaled_init(c, c->f32, c->u32, rA, c->p32, c->sc32);
-    k_set_trigger<<<1, 32, 0, st>>>(c->sc32, 1, delta2, 0.0);
+    k_set_trigger<<<1, 32, 0, st>>>(c->sc32, 1, delta2, 0.0, 1.0);
     c->launches += 2;
     double last_rec = 1.0;
     int cycles = 0, its = 0, done = 0, breakdowns = 0, slow = 0;
     bool finishFp64 = false, stalled = false;
     xdcg_status status = XDCG_NO_CONVERGENCE;
     while (true) {
-        s = scaled_iterate(c, c->u32, rA, rB, c->p32, c->q32, c->sc32, c->opt.max_iter, &its,
-                           &done, res, &stalled);
+        double rr = 0.0;
+        s = scaled_iterate(c, c->u32, rA, rB, c->p32, c->q32, c->sc32, c->opt.max_iter, its, &its,
+                           &done, &rr, res, &stalled);
         if (s != XDCG_OK) return s;
         if (done == kFault) return XDCG_TIMEOUT;
-        last_rec = std::sqrt(c->h_sc->rr);
+        last_rec = std::sqrt(rr);
         // fold the FP32 correction into u (FP64): u += L^-T u~ / s0
         launch_bwd_accum(c->nNodes, L.dofStart64, L.dofStart32, L.dofStart64, L.F, c->u32, 1.0 / s0,
                          u, st);
@@ -787,10 +866,13 @@ xdcg_status solve_mixed(xdcg_ctx *c, const double *f, double *u, double tol, boo
         // replace the recursive residual by the scaled true residual and finish
         // the interrupted iteration: z = r + Z~ nu, beta, p = z + beta p (beta =
         // 0 if the replacement moved the residual far: see k_coarse mode 3)
+        // (the stream is idle here: no launch queued past the stop can still
+        // report iteration its)
+        RunFollower::clear(c, its);
         float *rbuf = (c->userBlocks || !(its & 1)) ? rA : rB;
         launch_fwd_scale(c->nNodes, L.dofStart64, L.dofStart64, L.dofStart32, L.F, c->r64, s0, rbuf,
                          st);
-        k_set_trigger<<<1, 32, 0, st>>>(c->sc32, 0, 0.0, 0.0);
+        k_set_trigger<<<1, 32, 0, st>>>(c->sc32, 0, 0.0, 0.0, 1.0);
         if (c->userBlocks) {
             launch_update_plain<float>(nullptr, rbuf, nullptr, nullptr, c->n, 1, c->partials,
                                        c->sc32, st);
@@ -806,17 +888,13 @@ xdcg_status solve_mixed(xdcg_ctx *c, const double *f, double *u, double tol, boo
         launch_prolong_rows(L.R, c->nu32, c->userBlocks ? c->y32 : rbuf, c->p32,
                             done == kBreakdown ? 2 : 0, c->sc32, st);
         c->launches += 5;
-        CK(cudaMemcpyAsync(c->h_sc, c->sc32, sizeof(Scalars), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
         // next replacement: a further factor inner_tol, or sooner when the
         // scaled residual, at the ratio just observed between the scaled and
         // the true norm, should be at half the target -- but not before it has
         // dropped by a factor 10: near the target a few CG steps shorten the
         // scaled residual without shortening the true one
-        const double gamma2 = c->h_sc->rr / (s0 * s0 * rn2);
-        const double floor2 = std::min(0.25 * tol * tol * ff * s0 * s0 * gamma2,
-                                       kMinGroupDrop2 * c->h_sc->rr);
-        k_set_trigger<<<1, 32, 0, st>>>(c->sc32, 1, delta2, floor2);
+        k_set_trigger<<<1, 32, 0, st>>>(c->sc32, 1, delta2, 0.25 * tol * tol * ff * s0 * s0,
+                                        s0 * s0 * rn2);
         c->launches += 1;
     }
     res->iterations = its;
@@ -1271,8 +1349,7 @@ void free_ctx(xdcg_ctx *c) {
     if (c->h_sc) cudaFreeHost(c->h_sc);
     if (c->h_bs) cudaFreeHost(c->h_bs);
     if (c->h_slots) cudaFreeHost(c->h_slots);
-    if (c->h_done) cudaFreeHost(c->h_done);
-    if (c->h_poll) cudaFreeHost(c->h_poll);
+    if (c->h_prog) cudaFreeHost(c->h_prog);
     for (auto e : c->evS) cudaEventDestroy(e);
     for (auto e : c->evE) cudaEventDestroy(e);
     for (auto e : c->evP) cudaEventDestroy(e);
@@ -2474,8 +2551,7 @@ xdcg_status setup_impl(xdcg_ctx *c, const xdcg_matrix *K, const xdcg_deflation *
     CK(cudaMemsetAsync(c->sc32, 0, sizeof(Scalars), st));
     CK(cudaMemsetAsync(c->aux, 0, sizeof(Scalars), st));
     if (cudaMallocHost(&c->h_sc, sizeof(Scalars)) != cudaSuccess) return XDCG_OOM;
-    if (cudaMallocHost(&c->h_done, 2 * sizeof(int)) != cudaSuccess) return XDCG_OOM;
-    if (cudaMallocHost(&c->h_poll, 2 * sizeof(Scalars)) != cudaSuccess) return XDCG_OOM;
+    if (cudaMallocHost(&c->h_prog, sizeof(Progress)) != cudaSuccess) return XDCG_OOM;
     CK(cudaEventCreate(&c->ev0));
     CK(cudaEventCreate(&c->ev1));
     CK(cudaEventCreateWithFlags(&c->evb[0], cudaEventDisableTiming));

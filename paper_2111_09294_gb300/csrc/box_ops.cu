@@ -294,6 +294,7 @@ __device__ __forceinline__ void prolong_box(const BoxDev<double> &B, int s, int 
     };
     if (t < o1) load_node();
     pdl_wait();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) report(sc);
     if (sc->done != kRunning) return;
     if (t >= o1) return;
     const double beta = sc->beta;
@@ -759,6 +760,7 @@ __device__ __forceinline__ void prolong_rows_unit(const RowBoxDev &B, int unit,
     if (early) load();
     pdl_wait();
     if ((int)gridDim.x <= kTriggerBlocks) pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) report(sc);
     if (sc->done != kRunning) return;
     if (!early) load();
     const float beta = (float)sc->beta;

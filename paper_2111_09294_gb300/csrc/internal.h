@@ -25,6 +25,18 @@ enum Fin : int {
     kFinDefer = 3,   // each block's sum stored at partials[block]; the next kernel adds them
 };
 
+// What the host follows a run by, in pinned host memory that the device writes.
+// The prolongation that ends iteration its stores ||r||^2 in rr[its % kRing],
+// with the sign bit set once the run has stopped; stop (iterations and done
+// flag) is written before that.  A slot holds kNoReport until then: one 8-byte
+// store per iteration, no copy and no event in the stream.
+constexpr int kRing = 64;
+constexpr unsigned long long kNoReport = 0x7ff8dead00000000ull;   // a NaN no sum of squares gives
+struct Progress {
+    unsigned long long rr[kRing];
+    unsigned long long stop;   // its << 32 | done
+};
+
 // Scalars of one CG run, in device memory.  Written only by the last block
 // of a reduction kernel (single writer), read by all later kernels.
 struct Scalars {
@@ -43,6 +55,7 @@ struct Scalars {
     double *hist;     // if not null: ||r_i||^2 of iteration i, i < histCap
     int histCap;
     int pad2;
+    Progress *prog;   // if not null: where the prolongation reports each iteration
 };
 
 // Chunked 3x3 BSR over the chunk rows (3 consecutive dofs) in sliced-ELL

@@ -279,6 +279,22 @@ __device__ __forceinline__ bool grid_sum_t0(double v, double *partials, unsigned
     return true;
 }
 
+// Reports the run's state to the host (one thread of a kernel that ends an
+// iteration, after its wait; launches queued past a stop repeat the report).
+__device__ __forceinline__ void report(const Scalars *sc) {
+    volatile Progress *p = sc->prog;
+    if (!p) return;
+    unsigned long long v = (unsigned long long)__double_as_longlong(sc->rr);
+    if (sc->done == kRunning) {
+        if (sc->rr == 0.0) return;   // a prolongation before the first residual
+    } else {
+        p->stop = (unsigned long long)(unsigned int)sc->its << 32 | (unsigned int)sc->done;
+        __threadfence_system();
+        v |= 0x8000000000000000ull;
+    }
+    p->rr[sc->its % kRing] = v;
+}
+
 // Shared last-block actions on the scalar block.
 __device__ __forceinline__ void finalize(Scalars *sc, int fin, int slot, double val) {
     if (fin == kFinAlpha) {

@@ -55,3 +55,20 @@ def test_mixed_box_sizes(m, n_box):
     assert info["rel_res_true"] <= 1e-12
     assert np.linalg.norm(u.cpu().numpy() - ref.u) <= 1e-7 * np.linalg.norm(ref.u)
     s.close()
+
+
+# runs that end at every point of the host's look-ahead: the iteration cap at
+# each of its first iterations, FP64 and mixed, streams and recorded graphs
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("graph", [False, True])
+def test_iteration_caps(precision, graph):
+    from paper_2111_09294_gb300 import Solver
+    P = X.make("cube8_edge")
+    f = torch.tensor(P.f, device="cuda")
+    for cap in (0, 1, 2, 3, 4, 7, 8, 9, 17, 64):
+        s = Solver.from_problem(P, precision=precision, graph=graph, max_iter=cap)
+        _, info = s.solve(f, tol=1e-8, raise_on_error=False)
+        done = info["rel_res_true"] <= 1e-8
+        assert info["status"] == ("XDCG_OK" if done else "XDCG_NO_CONVERGENCE")
+        assert done == (cap == 64) and (done or info["iterations"] == cap)
+        s.close()

@@ -1399,8 +1399,9 @@ xdcg_status dense_inverse(xdcg_ctx *c, double *A, const std::vector<int> &dims,
     B.rowTileOff = upload_tmp(c, rowTileOff);
     B.cOff = upload_tmp(c, cOff);
     B.A = A;
-    B.D = dalloc_tmp<double>(c, (size_t)nMat * dense_inv_pivot_doubles());
-    B.C = dalloc_tmp<double>(c, (size_t)cTot);
+    B.D = dalloc_tmp<double>(c, 2 * (size_t)nMat * dense_inv_pivot_doubles());
+    B.C = dalloc_tmp<double>(c, 2 * (size_t)cTot);
+    B.cTotal = cTot;
     B.thr = dalloc_tmp<double>(c, nMat);
     B.bad = d_bad;
     B.badByMatrix = badByMatrix;

@@ -322,8 +322,8 @@ void launch_renumber(int nNodes, const int *nat, const int *in, const int *ot, c
 // nMat row-major matrices, matrix m (dim[m] x dim[m]) at A + off[m], inverted
 // in place.  Tile tables: rowTileOff = prefix of T_m, tileOff = prefix of
 // T_m (T_m + 1) / 2 (upper 64 x 64 tiles), T_m = ceil(dim[m] / 64).  Scratch:
-// D (nMat x 64 x 64), C (panel rows of matrix m at cOff[m], dim[m] x 64),
-// thr (nMat).  A pivot that is not above rel times the matrix's largest
+// D (2 x nMat x 64 x 64), C (two copies of cTotal: panel rows of matrix m at
+// cOff[m], dim[m] x 64), thr (nMat).  A pivot that is not above rel times the matrix's largest
 // diagonal entry sets *bad (atomic min) to the matrix index (badByMatrix) or
 // to the pivot's index within its matrix.
 struct DenseBatch {
@@ -333,6 +333,7 @@ struct DenseBatch {
     const int *tileOff, *rowTileOff;
     double *A, *D, *C, *thr;
     const long long *cOff;
+    long long cTotal;
     int *bad;
     int badByMatrix;
 };

@@ -52,36 +52,61 @@ __device__ __forceinline__ void z_row_of(const ZvalDev &Zv, int I, int j, int b,
     }
 }
 
+// Entry (j, c) of a node's deflation block (see z_row): by value, or from the
+// geometry without the rest of the row.
+__device__ __forceinline__ double z_entry(const ZvalDev &Zv, int J, int j, int b, int M, int menr,
+                                          const double *x, double H, int c) {
+    if (Zv.v) return Zv.v[Zv.off[J] + (long long)j * M + c];
+    if (j >= 3 && !(b == 6 && menr && c >= 6)) return 0.0;
+    const int a = j < 3 ? j : j - 3, c6 = c < 6 ? c : c - 6;
+    double r = 0.0;
+    if (c6 == a) r = 1.0;
+    if (a == 0) r = c6 == 4 ? x[2] : (c6 == 5 ? -x[1] : r);
+    if (a == 1) r = c6 == 3 ? -x[2] : (c6 == 5 ? x[0] : r);
+    if (a == 2) r = c6 == 3 ? x[1] : (c6 == 4 ? -x[0] : r);
+    return j < 3 && c >= 6 ? H * r : r;
+}
+
 // W block of entry e (node I coupled to box s): W_Is = sum_{J in s} K_IJ Z_J.
-__global__ void k_build_W(KinDev K, int nExt, const int *extBox, const int *extNode,
-                          const long long *wOff, const int *sub, const double *xrel,
-                          const signed char *hsign, const int *menr, ZvalDev Zv, double *W) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+// Eight threads per entry, each with three rows of one column at a time, the
+// sums in registers: about 1.8 ms at 32^3 (113k entries); one thread per entry
+// with its whole block in local memory took 7.3.
+constexpr int kWThreads = 8;
+
+__global__ void __launch_bounds__(128)
+k_build_W(KinDev K, int nExt, const int *extBox, const int *extNode, const long long *wOff,
+          const int *sub, const double *xrel, const signed char *hsign, const int *menr,
+          ZvalDev Zv, double *W) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int e = t / kWThreads;
     if (e >= nExt) return;
-    const int s = extBox[e], I = extNode[e];
-    const int M = menr[s] ? 12 : 6;
+    const int s = extBox[e], I = extNode[e], enr = menr[s];
+    const int M = enr ? 12 : 6;
     const int bI = K.dofStart[I + 1] - K.dofStart[I];
-    double acc[15 * 12];
-    for (int i = 0; i < bI * M; ++i) acc[i] = 0.0;
-    for (int p = K.rowPtr[I]; p < K.rowPtr[I + 1]; ++p) {
-        const int J = K.col[p];
-        if (sub[J] != s) continue;
-        const int bJ = K.dofStart[J + 1] - K.dofStart[J];
-        const double *Kb = K.val + K.valPtr[p];
-        const double X = xrel[3 * J], Y = xrel[3 * J + 1], Z = xrel[3 * J + 2];
-        const double H = (double)hsign[J];
-        for (int j = 0; j < bJ; ++j) {
-            double zr[12];
-            z_row_of(Zv, J, j, bJ, M, menr[s], X, Y, Z, H, zr);
-            for (int i = 0; i < bI; ++i) {
-                const double kij = Kb[i * bJ + j];
-                if (kij == 0.0) continue;
-                for (int c = 0; c < M; ++c) acc[i * M + c] += kij * zr[c];
+    const int p0 = K.rowPtr[I], p1 = K.rowPtr[I + 1];
+    double *Wb = W + wOff[e];
+    for (int task = t % kWThreads; task < bI / 3 * M; task += kWThreads) {
+        const int i0 = 3 * (task / M), c = task % M;
+        double acc[3] = {0.0, 0.0, 0.0};
+        for (int p = p0; p < p1; ++p) {
+            const int J = K.col[p];
+            if (sub[J] != s) continue;
+            const int bJ = K.dofStart[J + 1] - K.dofStart[J];
+            const double *Kb = K.val + K.valPtr[p] + (long long)i0 * bJ;
+            const double x[3] = {xrel[3 * J], xrel[3 * J + 1], xrel[3 * J + 2]};
+            const double H = (double)hsign[J];
+            for (int j = 0; j < bJ; ++j) {
+                const double z = z_entry(Zv, J, j, bJ, M, enr, x, H, c);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const double kij = Kb[(long long)i * bJ + j];
+                    if (kij != 0.0) acc[i] = fma(kij, z, acc[i]);
+                }
             }
         }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) Wb[(i0 + i) * M + c] = acc[i];
     }
-    double *Wb = W + wOff[e];
-    for (int i = 0; i < bI * M; ++i) Wb[i] = acc[i];
 }
 
 void launch_build_W(const KinDev &K, int nExt, const int *extBox, const int *extNode,
@@ -89,8 +114,9 @@ void launch_build_W(const KinDev &K, int nExt, const int *extBox, const int *ext
                     const signed char *hsign, const int *menr, const ZvalDev &Zv, double *W,
                     cudaStream_t st) {
     if (nExt == 0) return;
-    k_build_W<<<(nExt + 127) / 128, 128, 0, st>>>(K, nExt, extBox, extNode, wOff, sub, xrel,
-                                                   hsign, menr, Zv, W);
+    const long long threads = (long long)nExt * kWThreads;
+    k_build_W<<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(K, nExt, extBox, extNode, wOff,
+                                                                 sub, xrel, hsign, menr, Zv, W);
 }
 
 // E block (owner box t rows, box s columns) from one segment of box s's

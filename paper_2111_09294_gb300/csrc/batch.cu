@@ -90,11 +90,40 @@ __device__ __forceinline__ void batch_finalize(BatchScalars *bs, int m, int fin,
 }
 
 // ---- batched product Y = K~ X (+ x_j^T y_j, or ||y_j||^2 with y = b - K~ x) --
+//
+// A lane holds four columns, so MB = 8 gives two lanes to a slot of a step: a
+// pass takes 32 / LPS slots (LPS = MB / 4 lanes each) and a step LPS passes.
+// The lanes of a slot read whole 32-byte sectors of x (one lane with all eight
+// columns read 16 bytes from each of 24 cache lines per load, and the L1's tag
+// rate bounded the product), and the gather of the next pass is in flight
+// while this one is computed.  Stages run across slice boundaries, as in the
+// single product (k_spmv_lean); each row's terms are added in the order of its
+// slots, partial rows by the same tree.  8 columns at 32^3 (1.1M blocks): 41.5
+// us before, KSPMM now.
+// The warp's copy schedule (LeanWalk of the single product, step numbers in 32
+// bits: a step is 1,280 bytes).
+struct BatchWalk {
+    int pos, end, xPos, xEnd, isS;
+    __device__ __forceinline__ bool next(int C, int &sS, int &p, int &n) {
+        if (pos == end) {
+            if (!isS || xPos == xEnd) return false;
+            isS = 0;
+            pos = xPos;
+            end = xEnd;
+        }
+        sS = isS;
+        p = pos;
+        n = min(C, end - pos);
+        pos += n;
+        return true;
+    }
+};
 
 template <int MB, bool RES>
 __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nblk,
                                           unsigned char *smem) {
     constexpr int C = SpmvCfg<float, 0>::C, NS = SpmvCfg<float, 0>::NS, SB = stage_bytes<float, 0>();
+    constexpr int LPS = MB / 4, SPP = 32 / LPS;   // lanes per slot, slots per pass
     const SpmvDev<float> &A = args.A;
     const int m = args.m, fin = args.fin;
     const float *__restrict__ x = args.x;
@@ -102,59 +131,62 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
     float *__restrict__ y = args.y;
     BatchScalars *bs = args.bs;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int sl0 = lane / LPS, qc = lane % LPS;   // the lane's slot of pass 0, its columns / 4
     unsigned char *ring = smem + (size_t)warp * NS * SB;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kSpmvWarps * NS * SB) + warp * NS;
-    int *meta = reinterpret_cast<int *>(smem + (size_t)kSpmvWarps * NS * (SB + 8)) + warp * NS * 3;
     const int nS = A.S.nSlices;
     const int gw = blk * kSpmvWarps + warp;
-    const int sEnd = A.warpSlice[gw + 1];
+    const int sFirst = A.warpSlice[gw], sEnd = A.warpSlice[gw + 1];
     if (lane == 0) {
         for (int s = 0; s < NS; ++s) mbar_init(bars + s, 1);
         mbar_init_fence();
     }
+    // step counts of the warp's first 32 slices, and its two parts' step runs
+    __shared__ int tSteps[kSpmvWarps][32];
+    if (sFirst + lane < sEnd) {
+        const int g = sFirst + lane;
+        const SellDev<float> &P = g < nS ? A.S : A.X;
+        const int sl = g < nS ? g : g - nS;
+        tSteps[warp][lane] = (int)((P.slicePtr[sl + 1] - P.slicePtr[sl]) >> 5);
+    }
+    const int sA = min(sEnd, nS);
+    const int xa0 = max(sFirst, nS) - nS, xa1 = sEnd - nS;
+    BatchWalk pw;
+    pw.xPos = xa0 < xa1 ? (int)(A.X.slicePtr[xa0] >> 5) : 0;
+    pw.xEnd = xa0 < xa1 ? (int)(A.X.slicePtr[xa1] >> 5) : 0;
+    pw.isS = sFirst < sA;
+    pw.pos = pw.isS ? (int)(A.S.slicePtr[sFirst] >> 5) : pw.xPos;
+    pw.end = pw.isS ? (int)(A.S.slicePtr[sA] >> 5) : pw.xEnd;
+    BatchWalk cw = pw;
     __syncwarp();
     const uint64_t stream = l2_stream_policy();
     const unsigned long long deadline = global_ns() + A.waitNs;
-    int issued = 0, more = 1, pSlice = A.warpSlice[gw] - 1, pStep = 0, pSteps = 0;
-    long long pBase = 0;
-    const int *pCol = nullptr;
-    const float *pVal = nullptr;
+    int issued = 0, pslot = 0;
+    bool more = true;
     auto issue = [&]() {
-        if (pStep >= pSteps) {
-            if (++pSlice >= sEnd) {
-                more = 0;
-                return;
-            }
-            const bool isS = pSlice < nS;
-            const SellDev<float> &P = isS ? A.S : A.X;
-            const int sl = isS ? pSlice : pSlice - nS;
-            pBase = P.slicePtr[sl];
-            pSteps = (int)((P.slicePtr[sl + 1] - pBase) >> 5);
-            pStep = 0;
-            pCol = P.col;
-            pVal = P.val;
+        int sS, n, p;
+        if (!pw.next(C, sS, p, n)) {
+            more = false;
+            return;
         }
-        const int st = issued % NS;
-        const int n = min(C, pSteps - pStep);
-        meta[st * 3] = pSlice;
-        meta[st * 3 + 1] = pStep;
-        meta[st * 3 + 2] = n;
-        unsigned char *dst = ring + st * SB;
-        const uint32_t cb = (uint32_t)n * 128u, vb = (uint32_t)n * 288u * 4u;
-        const long long off = pBase + 32LL * pStep;
-        fence_proxy_async_smem();
-        mbar_arrive_expect_tx(bars + st, cb + vb);
-        bulk_g2s(dst, pCol + off, cb, bars + st, stream);
-        bulk_g2s(dst + C * 128, pVal + 9 * off, vb, bars + st, stream);
-        pStep += n;
+        if (lane == 0) {
+            const SellDev<float> &P = sS ? A.S : A.X;
+            unsigned char *dst = ring + pslot * SB;
+            fence_proxy_async_smem();
+            mbar_arrive_expect_tx(bars + pslot, (uint32_t)n * 1280u);
+            bulk_g2s(dst, P.col + 32LL * p, (uint32_t)n * 128u, bars + pslot, stream);
+            bulk_g2s(dst + C * 128, P.val + 288LL * p, (uint32_t)n * 1152u, bars + pslot, stream);
+        }
         ++issued;
+        pslot = pslot + 1 == NS ? 0 : pslot + 1;
     };
     // prologue copies before the wait unless the run has visibly stopped
     // (an L2 read that may be stale; the read after the wait decides)
-    const bool early = __ldcg(&bs->done) == kRunning && (fin != 0 || __ldcg(&bs->go));
-    if (lane == 0 && early)
+    const bool early = __shfl_sync(0xffffffffu,
+                                   __ldcg(&bs->done) == kRunning && (fin != 0 || __ldcg(&bs->go))
+                                       ? 1 : 0, 0) != 0;
+    if (early)
         while (more && issued < NS) issue();
-    issued = __shfl_sync(0xffffffffu, issued, 0);
     pdl_wait();
     if (!batch_runs(bs, fin == 0)) {
         const unsigned long long drain = global_ns() + kDrainNs;
@@ -162,122 +194,172 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
         __syncwarp();
         return;
     }
-    if (!early) {
-        if (lane == 0)
-            while (more && issued < NS) issue();
-        issued = __shfl_sync(0xffffffffu, issued, 0);
-    }
+    if (!early)
+        while (more && issued < NS) issue();
 
-    float part[MB];
+    float part[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    int sl = sFirst - 1, remS = 0, rpw = 16;
+    int row = -1;                 // the lane's chunk row, where it owns one
+    float a[LPS][3][4];           // [pass][row of the block][column]
 #pragma unroll
-    for (int j = 0; j < MB; ++j) part[j] = 0.0f;
-    int cur = -1, rpw = 16, rl = 0, h = 0;
-    bool valid = false, isS = true;
-    float a[3][MB];
+    for (int q = 0; q < LPS; ++q)
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+        for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < MB; ++j) a[i][j] = 0.0f;
+            for (int j = 0; j < 4; ++j) a[q][i][j] = 0.0f;
     auto finish = [&]() {
-        for (int o = rpw; o < 32; o <<= 1) {
+        // slot l of the 32 is lane l % SPP of pass l / SPP: slots 1 ... SPP / 2
+        // apart are LPS times as many lanes apart, slots SPP apart are passes
+        for (int o = rpw; o < SPP; o <<= 1)
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < MB; ++j) a[i][j] += __shfl_xor_sync(0xffffffffu, a[i][j], o);
-        }
-        if (valid && h == 0) {
-            const long long r3 = 3 * (long long)(isS ? A.S.row[rl] : A.X.row[rl]);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                float4 *yr = reinterpret_cast<float4 *>(y + (r3 + i) * MB);
-                const float4 *src = reinterpret_cast<const float4 *>(RES ? b : x) + (r3 + i) * (MB / 4);
-#pragma unroll
-                for (int q = 0; q < MB / 4; ++q) {
-                    const float4 s4 = src[q];
-                    float4 o4;
-                    if (RES) {
-                        o4 = make_float4(s4.x - a[i][4 * q], s4.y - a[i][4 * q + 1],
-                                         s4.z - a[i][4 * q + 2], s4.w - a[i][4 * q + 3]);
-                        part[4 * q] = fmaf(o4.x, o4.x, part[4 * q]);
-                        part[4 * q + 1] = fmaf(o4.y, o4.y, part[4 * q + 1]);
-                        part[4 * q + 2] = fmaf(o4.z, o4.z, part[4 * q + 2]);
-                        part[4 * q + 3] = fmaf(o4.w, o4.w, part[4 * q + 3]);
-                    } else {
-                        o4 = make_float4(a[i][4 * q], a[i][4 * q + 1], a[i][4 * q + 2],
-                                         a[i][4 * q + 3]);
-                        part[4 * q] = fmaf(s4.x, o4.x, part[4 * q]);
-                        part[4 * q + 1] = fmaf(s4.y, o4.y, part[4 * q + 1]);
-                        part[4 * q + 2] = fmaf(s4.z, o4.z, part[4 * q + 2]);
-                        part[4 * q + 3] = fmaf(s4.w, o4.w, part[4 * q + 3]);
-                    }
-                    yr[q] = o4;
-                }
-            }
-        }
-    };
-    int k = 0;
-    bool ok = true;
-    for (; k < issued; ++k) {
-        const int st = k % NS;
-        ok = __all_sync(0xffffffffu, mbar_wait(bars + st, (uint32_t)(k / NS) & 1u, deadline));
-        if (!ok) break;
-        const int sl = meta[st * 3], n = meta[st * 3 + 2];
-        if (sl != cur) {
-            if (cur >= 0) finish();
-            cur = sl;
-            isS = sl < nS;
-            rpw = isS ? 32 / kTprS : 32 / kTprX;
-            rl = (isS ? sl : sl - nS) * rpw + (lane % rpw);
-            h = lane / rpw;
-            valid = rl < (isS ? A.S.nRows : A.X.nRows);
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < MB; ++j) a[i][j] = 0.0f;
-        }
-        const int *cs = reinterpret_cast<const int *>(ring + st * SB);
-        const float *vs = reinterpret_cast<const float *>(ring + st * SB + C * 128);
-#pragma unroll
-        for (int t = 0; t < C; ++t) {
-            if (t < n) {
-                const int c = cs[t * 32 + lane];
-                const float4 *xc = reinterpret_cast<const float4 *>(x) + (size_t)c * (3 * MB / 4);
-                float xv[3][MB];
-#pragma unroll
-                for (int jc = 0; jc < 3; ++jc)
-#pragma unroll
-                    for (int q = 0; q < MB / 4; ++q) {
-                        const float4 v4 = __ldg(xc + jc * (MB / 4) + q);
-                        xv[jc][4 * q] = v4.x;
-                        xv[jc][4 * q + 1] = v4.y;
-                        xv[jc][4 * q + 2] = v4.z;
-                        xv[jc][4 * q + 3] = v4.w;
-                    }
-                const float *v = vs + t * 288 + lane;
+            for (int q = 0; q < LPS; ++q)
 #pragma unroll
                 for (int i = 0; i < 3; ++i)
 #pragma unroll
-                    for (int jc = 0; jc < 3; ++jc) {
-                        const float kv = v[(3 * i + jc) * 32];
+                    for (int j = 0; j < 4; ++j)
+                        a[q][i][j] += __shfl_xor_sync(0xffffffffu, a[q][i][j], o * LPS);
+        if (LPS == 2)
 #pragma unroll
-                        for (int j = 0; j < MB; ++j) a[i][j] = fmaf(kv, xv[jc][j], a[i][j]);
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) a[0][i][j] += a[LPS - 1][i][j];
+        if (row < 0) return;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const size_t at = ((size_t)row * 3 + i) * LPS + qc;
+            const float4 s4 = reinterpret_cast<const float4 *>(RES ? b : x)[at];
+            float4 o4;
+            if (RES) {
+                o4 = make_float4(s4.x - a[0][i][0], s4.y - a[0][i][1], s4.z - a[0][i][2],
+                                 s4.w - a[0][i][3]);
+                part[0] = fmaf(o4.x, o4.x, part[0]);
+                part[1] = fmaf(o4.y, o4.y, part[1]);
+                part[2] = fmaf(o4.z, o4.z, part[2]);
+                part[3] = fmaf(o4.w, o4.w, part[3]);
+            } else {
+                o4 = make_float4(a[0][i][0], a[0][i][1], a[0][i][2], a[0][i][3]);
+                part[0] = fmaf(s4.x, o4.x, part[0]);
+                part[1] = fmaf(s4.y, o4.y, part[1]);
+                part[2] = fmaf(s4.z, o4.z, part[2]);
+                part[3] = fmaf(s4.w, o4.w, part[3]);
+            }
+            reinterpret_cast<float4 *>(y)[at] = o4;
+        }
+    };
+    auto next_slice = [&]() {
+        if (sl >= sFirst) finish();
+        ++sl;
+        const bool isS = sl < nS;
+        rpw = isS ? 32 / kTprS : 32 / kTprX;
+        const int ls = isS ? sl : sl - nS;
+        const int rl = ls * rpw + sl0;
+        row = sl0 < rpw && rl < (isS ? A.S.nRows : A.X.nRows)
+                  ? (isS ? A.S.row[rl] : A.X.row[rl]) : -1;
+#pragma unroll
+        for (int q = 0; q < LPS; ++q)
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) a[q][i][j] = 0.0f;
+        if (sl - sFirst < 32) {
+            remS = tSteps[warp][sl - sFirst];
+        } else {
+            const SellDev<float> &P = isS ? A.S : A.X;
+            remS = (int)((P.slicePtr[ls + 1] - P.slicePtr[ls]) >> 5);
+        }
+    };
+    // x of the lane's slot of pass q of step t of the stage in ring slot st
+    auto gather = [&](int st, int t, int q, float4 (&xv)[3]) {
+        const int c = reinterpret_cast<const int *>(ring + st * SB)[t * 32 + q * SPP + sl0];
+        const float4 *xc = reinterpret_cast<const float4 *>(x) + (size_t)c * (3 * LPS) + qc;
+#pragma unroll
+        for (int jc = 0; jc < 3; ++jc) xv[jc] = __ldg(xc + jc * LPS);
+    };
+    int sS, cP, curN = 0, cslot = 0, consumed = 0;
+    uint32_t cpar = 0u;
+    bool ok = true, have = cw.next(C, sS, cP, curN);
+    float4 xn[3];
+    if (have) {
+        ok = __all_sync(0xffffffffu, mbar_wait(bars, 0u, deadline));
+        if (ok) gather(0, 0, 0, xn);
+    }
+    while (ok && have) {
+        int nxtN = 0;
+        const bool haveN = cw.next(C, sS, cP, nxtN);
+        const int nslot = cslot + 1 == NS ? 0 : cslot + 1;
+        const uint32_t npar = nslot == 0 ? cpar ^ 1u : cpar;
+        const float *vs = reinterpret_cast<const float *>(ring + cslot * SB + C * 128);
+#pragma unroll
+        for (int t = 0; t < C; ++t) {
+            if (t < curN && ok) {
+                if (remS == 0) next_slice();
+                --remS;
+#pragma unroll
+                for (int q = 0; q < LPS; ++q) {
+                    float4 xc[3] = {xn[0], xn[1], xn[2]};
+                    // the next pass: of this step, of the next, or of the next stage
+                    if (q + 1 < LPS) {
+                        gather(cslot, t, q + 1, xn);
+                    } else if (t + 1 < C && t + 1 < curN) {
+                        gather(cslot, t + 1, 0, xn);
+                    } else if (haveN) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(bars + nslot, npar, deadline));
+                        if (ok) gather(nslot, 0, 0, xn);
                     }
+                    const float *v = vs + t * 288 + q * SPP + sl0;
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+#pragma unroll
+                        for (int jc = 0; jc < 3; ++jc) {
+                            const float kv = v[(3 * i + jc) * 32];
+                            a[q][i][0] = fmaf(kv, xc[jc].x, a[q][i][0]);
+                            a[q][i][1] = fmaf(kv, xc[jc].y, a[q][i][1]);
+                            a[q][i][2] = fmaf(kv, xc[jc].z, a[q][i][2]);
+                            a[q][i][3] = fmaf(kv, xc[jc].w, a[q][i][3]);
+                        }
+                }
             }
         }
+        if (!ok) break;
         __syncwarp();
-        if (lane == 0 && more) issue();
-        issued = __shfl_sync(0xffffffffu, issued, 0);
+        if (more) issue();
+        ++consumed;
+        cslot = nslot;
+        cpar = npar;
+        curN = nxtN;
+        have = haveN;
     }
     if (ok) {
-        if (cur >= 0) finish();
+        if (sl >= sFirst) finish();
     } else {
+        // a copy did not land in time: flag it, give the copies still in
+        // flight a bounded chance to land, and leave the shared memory
         if (lane == 0) atomicExch(&bs->fault, 1);
         const unsigned long long drain = global_ns() + kDrainNs;
-        for (; k < issued; ++k) mbar_wait(bars + k % NS, (uint32_t)(k / NS) & 1u, drain);
+        for (int k = consumed; k < issued; ++k)
+            mbar_wait(bars + k % NS, (uint32_t)(k / NS) & 1u, drain);
         __syncwarp();
     }
+    // the block's sums: rows sit in slots 0 .. 15 of pass 0, so the trees over
+    // the 32 slots start eight slots apart
+    __shared__ float wsum[MB][kSpmvWarps];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+            part[j] += __shfl_xor_sync(0xffffffffu, part[j], o * LPS);
+        if (lane < LPS) wsum[4 * lane + j][warp] = part[j];
+    }
+    __syncthreads();
+    double blkSum = 0.0;
+    if (threadIdx.x < MB) {
+        float w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = wsum[threadIdx.x][i];
+        blkSum = (double)sum_of_8(w);
+    }
     double tot[MB];
-    if (grid_sum_of<float, MB>(part, args.partials, &bs->ticket[0], tot, blk, nblk) &&
+    if (grid_sum_lanes<MB>(blkSum, args.partials, &bs->ticket[0], tot, blk, nblk) &&
         threadIdx.x == 0) {
         if (bs->fault)
             bs->done = kFault;

@@ -953,7 +953,7 @@ RestrictBArgs restrict_args(xdcg_ctx *c, int m, int mode) {
 }
 CoarseBArgs coarse_args(xdcg_ctx *c, int m, int mode) {
     return CoarseBArgs{c->Einv32, c->bG32, c->k, m, mode, g_ld(c), mode == 0 ? nullptr : c->bZR,
-                       c->bNU, c->partials, c->bNU32, c->bs, c->L32.A.waitNs};
+                       c->bNU, c->partials, c->bNU32, c->bs};
 }
 ProlongBArgs prolong_args(xdcg_ctx *c, int m, int mode) {
     return ProlongBArgs{c->L32.Rb, m, mode, c->bNU32, c->bRA, c->bRB,

@@ -55,37 +55,44 @@ __device__ __forceinline__ int sys_of(const int *__restrict__ off, int nSys, int
 
 // ---- per-column scalar updates ----------------------------------------------
 
+// One column per lane (the divisions of a column are a chain of FP64
+// instructions of 64 cycles each, which eight lanes share); every lane of a
+// warp calls it, with column j's total in lane j.
+//
 // fin 0 (iteration): pq_j, alpha_j for the running columns (0 for the
 // others); a running column whose p^T K p is not positive is held as broken.
 // The iteration counts (its, its_j) advance when a column still runs;
 // otherwise the system stops until the host's next replacement.
 // fin 1 (start): rr_j.
-__device__ __forceinline__ void batch_finalize(BatchScalars *bs, int m, int fin,
-                                               const double *tot) {
-    if (fin == 0) {
-        bool any = false;
-        for (int j = 0; j < m; ++j) {
-            bs->pq[j] = tot[j];
-            if (!col_runs(bs, j, m)) {
-                bs->alpha[j] = 0.0;
-                continue;
-            }
+__device__ __forceinline__ void batch_finalize(BatchScalars *bs, int m, int fin, double tot) {
+    const int j = threadIdx.x & 31;
+    if (fin != 0) {
+        if (j < m) bs->rr[j] = tot;
+        return;
+    }
+    bool any = false;
+    if (j < m) {
+        bs->pq[j] = tot;
+        if (!col_runs(bs, j, m)) {
+            bs->alpha[j] = 0.0;
+        } else {
             bs->itsc[j] += 1;
-            if (!(tot[j] > 0.0) || !isfinite(tot[j])) {
+            if (!(tot > 0.0) || !isfinite(tot)) {
                 bs->alpha[j] = 0.0;
                 bs->broken[j] = 1;
                 bs->pend[j] = 1;
             } else {
-                bs->alpha[j] = bs->rho[j] / tot[j];
+                bs->alpha[j] = bs->rho[j] / tot;
                 any = true;
             }
         }
+    }
+    any = __any_sync(0xffffffffu, any);
+    if (j == 0) {
         if (any)
             bs->its += 1;
         else
             bs->done = kConverged;
-    } else {
-        for (int j = 0; j < m; ++j) bs->rr[j] = tot[j];
     }
 }
 
@@ -99,7 +106,7 @@ __device__ __forceinline__ void batch_finalize(BatchScalars *bs, int m, int fin,
 // while this one is computed.  Stages run across slice boundaries, as in the
 // single product (k_spmv_lean); each row's terms are added in the order of its
 // slots, partial rows by the same tree.  8 columns at 32^3 (1.1M blocks): 41.5
-// us before, 32.7 now.
+// us before, 29.9 now.
 // The warp's copy schedule (LeanWalk of the single product, step numbers in 32
 // bits: a step is 1,280 bytes).
 struct BatchWalk {
@@ -358,13 +365,13 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
         for (int i = 0; i < 8; ++i) w[i] = wsum[threadIdx.x][i];
         blkSum = (double)sum_of_8(w);
     }
-    double tot[MB];
+    double tot;
     if (grid_sum_lanes<MB>(blkSum, args.partials, &bs->ticket[0], tot, blk, nblk) &&
-        threadIdx.x == 0) {
-        if (bs->fault)
-            bs->done = kFault;
-        else
+        threadIdx.x < 32) {
+        if (!bs->fault)
             batch_finalize(bs, m, fin, tot);
+        else if (threadIdx.x == 0)
+            bs->done = kFault;
     }
 }
 
@@ -488,7 +495,8 @@ __device__ __forceinline__ void row_times(const float *z, float rn, float *acc) 
 // The unit's rows of Z~ and W~ and its dof map, shared by the columns, are
 // copied into shared memory before the wait for the product (set-up data);
 // four rows' entries of r, q, p and u are in flight at a time.  8 columns at
-// 32^3 (599 units): 30.4 us before, 23.2 now.
+// 32^3 (599 units): 30.4 us before, 18.6 now (four blocks
+// per SM).
 template <int MB, int M>
 __device__ __forceinline__ bool restrict_b_unit(const RestrictBArgs &a, int unit, float *stage,
                                                 float *rrs) {
@@ -645,35 +653,36 @@ __device__ __forceinline__ void restrict_b_body(const RestrictBArgs &a, int blk,
     if (!went || mode == 2) return;
     // lane j of warp 0 adds column j's ||r||^2
     const double rr = threadIdx.x < MB ? (double)rrs[threadIdx.x] : 0.0;
-    double tot[MB];
-    if (grid_sum_lanes<MB>(rr, a.partials, &bs->ticket[2], tot, blk, nblk) && threadIdx.x == 0) {
+    double tot;
+    if (grid_sum_lanes<MB>(rr, a.partials, &bs->ticket[2], tot, blk, nblk) && threadIdx.x < 32) {
+        const int j = threadIdx.x;   // one column per lane
         if (mode == 1) {
-            for (int j = 0; j < m; ++j)
-                if (bs->repl[j]) bs->rr[j] = tot[j];
+            if (j < m && bs->repl[j]) bs->rr[j] = tot;
             return;
         }
         bool any = false;
-        for (int j = 0; j < m; ++j) {
-            if (!col_runs(bs, j, m)) continue;
-            bs->rr[j] = tot[j];
-            if (tot[j] <= bs->trig[j] || !isfinite(tot[j])) bs->pend[j] = 1;
+        if (j < m && col_runs(bs, j, m)) {
+            bs->rr[j] = tot;
+            bool hold = tot <= bs->trig[j] || !isfinite(tot);
             if (bs->itsc[j] >= bs->max_it) {
-                bs->pend[j] = 1;
+                hold = true;
                 bs->last[j] = 1;
             }
-            any |= !bs->pend[j];
+            if (hold) bs->pend[j] = 1;
+            any = !hold;
         }
-        if (!any) bs->done = kConverged;
+        any = __any_sync(0xffffffffu, any);
+        if (j == 0 && !any) bs->done = kConverged;
     }
 }
 
 template <int MB>
-__global__ void __launch_bounds__(kThreads) k_restrict_b(RestrictBArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) k_restrict_b(RestrictBArgs a) {
     restrict_b_body<MB>(a, (int)blockIdx.x, (int)gridDim.x);
 }
 
 template <int MB>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 k_restrict_b_sys(const RestrictBArgs *__restrict__ tab, const int *__restrict__ off, int nSys) {
     const int s = sys_of(off, nSys, (int)blockIdx.x);
     const int b0 = __ldg(off + s);
@@ -710,12 +719,7 @@ __device__ __forceinline__ void lane_reduce_scatter(float (&v)[NV], int lane) {
 // sums per lane)
 template <int MB>
 __host__ __device__ constexpr int coarse_rows_b() { return 32 / MB; }
-constexpr int kCoarseChunkB = 128;   // columns of G per staged chunk (4 per lane)
-template <int MB>
-constexpr int coarse_smem_b() {
-    return kWarps * 2 * MB * kCoarseChunkB * (int)sizeof(float) +
-           kWarps * 2 * (int)sizeof(uint64_t);
-}
+constexpr int kCoarseChunkB = 128;   // columns of G per chunk (4 per lane)
 
 // One chunk's entries of E^-1 for a lane: 4 consecutive columns (one 16-byte
 // load per row, V = 4) or 4 columns 32 apart (V = 1) of each of the RB rows.
@@ -747,84 +751,55 @@ __device__ __forceinline__ void coarse_load_e(const float *Eb, int k, int rLast,
 // column that leaves, that broke down or whose residual the replacement
 // lengthened by more than 2x.  A block takes 32 / MB consecutive rows of
 // E^-1 and its warps split the columns into segments (multiples of 4).  Each
-// warp walks its segment in chunks of kCoarseChunkB columns: the chunk's
-// part of G (stored column by column) is staged in shared memory by bulk
-// copies, double-buffered (the next chunk's copy is in flight while this one
-// is used), and the lane's entries of E^-1 are loaded before the wait for
-// the chunk's copy (the first chunk's before the wait for the previous
-// kernel: E^-1 does not depend on it), so a chunk costs one memory round
-// trip.  The partial sums are reduced over the lanes, then over the warps in
-// order.
+// warp walks its segment in chunks of kCoarseChunkB columns (the first chunk's
+// entries of E^-1 loaded before the wait for the restriction: E^-1 does not
+// depend on it); G, stored column by column, is read through L1, where the SM's
+// blocks find it after the first.  The partial sums are reduced over the lanes,
+// then over the warps in order.  8 columns, k =
+// 3150: 29.9 us before (G staged by each warp in shared memory through bulk
+// copies and barriers), 24.2 now (three blocks of 80 registers per SM; four of 64
+// spill, 39).
 template <int MB, int V>
-__device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int nblk,
-                                              unsigned char *smem) {
+__device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int nblk) {
     constexpr int RB = coarse_rows_b<MB>(), NV = RB * MB, P = NV / 32, CH = kCoarseChunkB;
     __shared__ float red[kWarps][NV];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *gs = reinterpret_cast<float *>(smem) + (size_t)warp * 2 * MB * CH;   // [2][MB][CH]
-    uint64_t *bar =
-        reinterpret_cast<uint64_t *>(smem + (size_t)kWarps * 2 * MB * CH * sizeof(float)) +
-        2 * warp;
-    if (lane == 0) {
-        mbar_init(bar, 1);
-        mbar_init(bar + 1, 1);
-        mbar_init_fence();
-    }
-    __syncwarp();
     const int k = a.k;
     const int i0 = blk * RB;
     const int seg = (k + 4 * kWarps - 1) / (4 * kWarps) * 4;
     const int l0 = warp * seg, l1 = min(k, l0 + seg);
-    const int nch = l1 > l0 ? (l1 - l0 + CH - 1) / CH : 0;
     const uint64_t keep = l2_keep_policy();
     const float *Eb = a.Einv + (size_t)i0 * k;
     const int rLast = k - 1 - i0;
     float e[RB][4];
-    if (nch > 0) coarse_load_e<RB, V>(Eb, k, rLast, l0, min(CH, l1 - l0), lane, keep, e);
+    if (l0 < l1) coarse_load_e<RB, V>(Eb, k, rLast, l0, min(CH, l1 - l0), lane, keep, e);
     pdl_wait();
     BatchScalars *bs = a.bs;
     if (!batch_runs(bs, a.mode == 2)) return;
     const int m = a.m, mode = a.mode;
-    const unsigned long long deadline = global_ns() + a.waitNs;
-    auto issue = [&](int c) {   // lane 0: chunk c of G into buffer c & 1
-        const int lc = l0 + c * CH, cpad = (min(CH, l1 - lc) + 3) & ~3;
-        float *dst = gs + (c & 1) * MB * CH;
-        fence_proxy_async_smem();
-        mbar_arrive_expect_tx(bar + (c & 1), (uint32_t)(MB * cpad * sizeof(float)));
-#pragma unroll
-        for (int j = 0; j < MB; ++j)
-            bulk_g2s(dst + j * CH, a.G32 + (size_t)j * a.gld + lc, (uint32_t)(cpad * sizeof(float)),
-                     bar + (c & 1), keep);
-    };
     float acc[NV];
 #pragma unroll
     for (int t = 0; t < NV; ++t) acc[t] = 0.0f;
-    if (lane == 0 && nch > 0) issue(0);
-    int c = 0;
-    bool ok = true;
-    for (; c < nch; ++c) {
-        if (lane == 0 && c + 1 < nch) issue(c + 1);
-        const int lc = l0 + c * CH, clen = min(CH, l1 - lc);
-        if (c > 0) coarse_load_e<RB, V>(Eb, k, rLast, lc, clen, lane, keep, e);
-        ok = __all_sync(0xffffffffu, mbar_wait(bar + (c & 1), (uint32_t)(c >> 1) & 1u, deadline));
-        if (!ok) break;
-        const float *g0 = gs + (c & 1) * MB * CH;
+    for (int lc = l0; lc < l1; lc += CH) {
+        const int clen = min(CH, l1 - lc);
+        if (lc > l0) coarse_load_e<RB, V>(Eb, k, rLast, lc, clen, lane, keep, e);
+        const float *g0 = a.G32 + lc;
 #pragma unroll
         for (int j = 0; j < MB; ++j) {
-            float g[4];
-            // entries past the chunk are never read (shared memory there may
-            // hold anything, and 0 * NaN is NaN)
+            float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
             if (V == 4) {
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (4 * lane < clen) v = *reinterpret_cast<const float4 *>(g0 + j * CH + 4 * lane);
-                g[0] = v.x;
-                g[1] = v.y;
-                g[2] = v.z;
-                g[3] = v.w;
+                if (4 * lane < clen) {
+                    const float4 v =
+                        __ldg(reinterpret_cast<const float4 *>(g0 + (size_t)j * a.gld + 4 * lane));
+                    g[0] = v.x;
+                    g[1] = v.y;
+                    g[2] = v.z;
+                    g[3] = v.w;
+                }
             } else {
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    g[q] = lane + 32 * q < clen ? g0[j * CH + lane + 32 * q] : 0.0f;
+                    if (lane + 32 * q < clen) g[q] = __ldg(g0 + (size_t)j * a.gld + lane + 32 * q);
             }
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
@@ -834,14 +809,6 @@ __device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int
                 acc[r * MB + j] = fmaf(e[r][3], g[3], t);
             }
         }
-        __syncwarp();   // the buffer is read before a later copy overwrites it
-    }
-    if (!ok) {
-        // copies in flight (chunks c and c + 1) land before the block leaves
-        const unsigned long long drain = global_ns() + kDrainNs;
-        for (int d = c; d < min(nch, c + 2); ++d) mbar_wait(bar + (d & 1), (uint32_t)(d >> 1) & 1u, drain);
-        __syncwarp();
-        if (lane == 0) atomicExch(&bs->fault, 1);
     }
     lane_reduce_scatter<NV>(acc, lane);
 #pragma unroll
@@ -864,44 +831,40 @@ __device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int
 #pragma unroll
         for (int o = MB; o < 32; o <<= 1) pj += __shfl_xor_sync(0xffffffffu, pj, o);
     }
-    double tot[MB];
-    if (grid_sum_lanes<MB>(pj, a.partials, &bs->ticket[3], tot, blk, nblk) && threadIdx.x == 0) {
+    double tot;
+    if (grid_sum_lanes<MB>(pj, a.partials, &bs->ticket[3], tot, blk, nblk) && threadIdx.x < 32) {
+        const int j = threadIdx.x;   // one column per lane
         if (bs->fault) {
-            bs->done = kFault;
-        } else if (mode != 0) {
-            for (int j = 0; j < m; ++j) {
-                const bool upd = mode == 2 ? col_runs(bs, j, m) : (mode == 1 || bs->repl[j]);
-                if (!upd) continue;
-                const double rho_new = bs->rr[j] + tot[j];
-                if (mode == 1 || !bs->active[j] ||
-                    (mode == 3 && (bs->broken[j] || bs->rr[j] > 4.0 * bs->rrRep[j])))
-                    bs->beta[j] = 0.0;
-                else
-                    bs->beta[j] = rho_new / bs->rho[j];
-                bs->rho[j] = rho_new;
-                if (mode == 3) bs->broken[j] = 0;
-            }
+            if (j == 0) bs->done = kFault;
+        } else if (mode != 0 && j < m &&
+                   (mode == 2 ? col_runs(bs, j, m) : (mode == 1 || bs->repl[j]))) {
+            const double rho_new = bs->rr[j] + tot;
+            if (mode == 1 || !bs->active[j] ||
+                (mode == 3 && (bs->broken[j] || bs->rr[j] > 4.0 * bs->rrRep[j])))
+                bs->beta[j] = 0.0;
+            else
+                bs->beta[j] = rho_new / bs->rho[j];
+            bs->rho[j] = rho_new;
+            if (mode == 3) bs->broken[j] = 0;
         }
     }
 }
 
 template <int MB, int V>
 __global__ void __launch_bounds__(kThreads, MB == 8 ? 3 : 2) k_coarse_b(CoarseBArgs a) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    coarse_b_body<MB, V>(a, (int)blockIdx.x, (int)gridDim.x, smem);
+    coarse_b_body<MB, V>(a, (int)blockIdx.x, (int)gridDim.x);
 }
 
 template <int MB>
 __global__ void __launch_bounds__(kThreads, MB == 8 ? 3 : 2)
 k_coarse_b_sys(const CoarseBArgs *__restrict__ tab, const int *__restrict__ off, int nSys) {
-    extern __shared__ __align__(128) unsigned char smem[];
     const int s = sys_of(off, nSys, (int)blockIdx.x);
     const int b0 = __ldg(off + s), nb = __ldg(off + s + 1) - b0;
     const CoarseBArgs &a = tab[s];
     if ((a.k & 3) == 0)
-        coarse_b_body<MB, 4>(a, (int)blockIdx.x - b0, nb, smem);
+        coarse_b_body<MB, 4>(a, (int)blockIdx.x - b0, nb);
     else
-        coarse_b_body<MB, 1>(a, (int)blockIdx.x - b0, nb, smem);
+        coarse_b_body<MB, 1>(a, (int)blockIdx.x - b0, nb);
 }
 
 int coarse_b_blocks(int k, int MB) {
@@ -913,7 +876,7 @@ int coarse_b_blocks(int k, int MB) {
 template <int MB>
 void launch_coarse_b(const CoarseBArgs &a, cudaStream_t st) {
     launch_pdl(a.k % 4 == 0 ? k_coarse_b<MB, 4> : k_coarse_b<MB, 1>, coarse_b_blocks(a.k, MB),
-               kThreads, coarse_smem_b<MB>(), st, a);
+               kThreads, 0, st, a);
 }
 
 // ---- batched prolongation -----------------------------------------------------
@@ -1034,8 +997,7 @@ void launch_iteration_sys(const BatchSysTab &t, cudaStream_t st) {
     const int smem = spmv_smem_bytes<float, 0>();
     launch_pdl(k_spmm_sys<MB>, t.blocks[0], kSpmvThreads, smem, st, t.spmm, t.off[0], t.nSys);
     launch_pdl(k_restrict_b_sys<MB>, t.blocks[1], kThreads, kStageBytesB, st, t.rst, t.off[1], t.nSys);
-    launch_pdl(k_coarse_b_sys<MB>, t.blocks[2], kThreads, coarse_smem_b<MB>(), st, t.crs, t.off[2],
-               t.nSys);
+    launch_pdl(k_coarse_b_sys<MB>, t.blocks[2], kThreads, 0, st, t.crs, t.off[2], t.nSys);
     launch_pdl(k_prolong_b_sys<MB>, t.blocks[3], kThreads, 0, st, t.pro, t.off[3], t.nSys);
 }
 
@@ -1226,13 +1188,7 @@ bool spmm_prepare() {
     const int smem = spmv_smem_bytes<float, 0>();
     return set_smem(k_spmm<4, false>, smem) && set_smem(k_spmm<4, true>, smem) &&
            set_smem(k_spmm<8, false>, smem) && set_smem(k_spmm<8, true>, smem) &&
-           set_smem(k_spmm_sys<4>, smem) && set_smem(k_spmm_sys<8>, smem) &&
-           set_smem(k_coarse_b<4, 4>, coarse_smem_b<4>()) &&
-           set_smem(k_coarse_b<4, 1>, coarse_smem_b<4>()) &&
-           set_smem(k_coarse_b<8, 4>, coarse_smem_b<8>()) &&
-           set_smem(k_coarse_b<8, 1>, coarse_smem_b<8>()) &&
-           set_smem(k_coarse_b_sys<4>, coarse_smem_b<4>()) &&
-           set_smem(k_coarse_b_sys<8>, coarse_smem_b<8>());
+           set_smem(k_spmm_sys<4>, smem) && set_smem(k_spmm_sys<8>, smem);
 }
 
 #define XDCG_BATCH_INST(MB)                                                                    \

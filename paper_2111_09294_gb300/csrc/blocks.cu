@@ -142,8 +142,8 @@ k_block_apply(BlkDev<T> B, const T *__restrict__ r, T *__restrict__ y, double *p
             part[0] = fma(rs[i], s, part[0]);
         }
     }
-    double tot[1];
-    if (grid_sum<T, 1>(part, partials, &sc->ticket[1], tot) && threadIdx.x == 0) sc->ry = tot[0];
+    double tot;
+    if (grid_sum<T>(part[0], partials, &sc->ticket[1], tot) && threadIdx.x == 0) sc->ry = tot;
 }
 
 template <typename T>
@@ -176,15 +176,15 @@ k_update_plain(T *u, T *r, const T *p, const T *q, long long n, int mode, double
         }
         v[0] = fma(ri, ri, v[0]);
     }
-    double tot[1];
-    if (grid_sum<T, 1>(v, partials, &sc->ticket[2], tot) && threadIdx.x == 0) {
-        sc->rr = tot[0];
-        if (sc->hist && sc->its < sc->histCap) sc->hist[sc->its] = tot[0];
-        if (tot[0] <= sc->tol2ff)
+    double tot;
+    if (grid_sum<T>(v[0], partials, &sc->ticket[2], tot) && threadIdx.x == 0) {
+        sc->rr = tot;
+        if (sc->hist && sc->its < sc->histCap) sc->hist[sc->its] = tot;
+        if (tot <= sc->tol2ff)
             sc->done = kConverged;
         else if (sc->its >= sc->max_it)
             sc->done = kMaxIter;
-        else if (!isfinite(tot[0]))
+        else if (!isfinite(tot))
             sc->done = kBreakdown;
     }
 }

@@ -446,7 +446,6 @@ struct CoarseBArgs {
     double *NU, *partials;
     float *NU32;
     BatchScalars *bs;
-    unsigned long long waitNs; // limit of the bounded waits on the bulk copies of G
 };
 struct ProlongBArgs {
     RowBoxDev B;

@@ -210,8 +210,9 @@ k_update(NodeDev<double> N, double *u, double *r, const double *p, const double 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double tot[2];
-    sum_partials<2>(partials, &sc->ticket[2], tot, nUnits);
+    const double sum = sum_partials<2>(partials, &sc->ticket[2], nUnits);
+    if (warp != 0) return;
+    const double tot[2] = {sum, __shfl_sync(0xffffffffu, sum, 1)};
     if (threadIdx.x == 0) {
         sc->ry = tot[1];
         sc->rr = tot[0];

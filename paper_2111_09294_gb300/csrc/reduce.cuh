@@ -89,10 +89,10 @@ __device__ __forceinline__ float sum_of_8(const float (&x)[8]) {
 // partials (partials[i * nblk + b]) added by one warp, its lanes striding
 // over the blocks with four accumulators each, then across the lanes (a fixed
 // order, and FP64 work spread over the warps: FP64 arithmetic is slow here).
-// Thread 0 gets the totals and resets the ticket.
+// Thread i < NV gets total i; thread 0 resets the ticket.
 template <int NV>
-__device__ __forceinline__ void sum_partials(const double *partials, unsigned int *ticket,
-                                             double (&tot)[NV], int nblk) {
+__device__ __forceinline__ double sum_partials(const double *partials, unsigned int *ticket,
+                                               int nblk) {
     __shared__ double fin[NV];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int i = w; i < NV; i += nw) {
@@ -112,19 +112,19 @@ __device__ __forceinline__ void sum_partials(const double *partials, unsigned in
         if (l == 0) fin[i] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int i = 0; i < NV; ++i) tot[i] = fin[i];
-        *ticket = 0u;
-    }
+    if (threadIdx.x == 0) *ticket = 0u;
+    return threadIdx.x < NV ? fin[threadIdx.x] : 0.0;
 }
 
 // Grid-wide sum of NV <= 32 values whose block totals lanes 0 .. NV - 1 of
-// warp 0 already hold (one per lane, in v): as grid_sum_of without the block
-// reduction.  Every thread of the block calls it.
+// warp 0 already hold (one per lane, in v): as grid_sum without the block
+// reduction, over the blocks blk = 0 .. nblk - 1 of one reduction (the launch's, or
+// one system's share of a launch over several systems); in the last block to
+// finish, which returns true, the totals come back to the same lanes.  Every
+// thread of the block calls it.  partials: NV * nblk doubles.
 template <int NV>
 __device__ __forceinline__ bool grid_sum_lanes(double v, double *partials, unsigned int *ticket,
-                                               double (&tot)[NV], int blk, int nblk) {
+                                               double &tot, int blk, int nblk) {
     __shared__ bool last;
     if (threadIdx.x < 32) {
         if ((int)threadIdx.x < NV) partials[(size_t)threadIdx.x * nblk + blk] = v;
@@ -135,30 +135,7 @@ __device__ __forceinline__ bool grid_sum_lanes(double v, double *partials, unsig
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    sum_partials<NV>(partials, ticket, tot, nblk);
-    return true;
-}
-
-// Sum over the blocks blk = 0 .. nblk - 1 of one reduction (the launch's
-// blocks, or one system's share of a launch over several systems).  Returns
-// true in exactly one of them (the last to finish), where thread 0 then holds
-// the FP64 totals in tot.  partials: NV * nblk doubles.
-template <typename A, int NV>
-__device__ __forceinline__ bool grid_sum_of(A (&v)[NV], double *partials, unsigned int *ticket,
-                                            double (&tot)[NV], int blk, int nblk) {
-    __shared__ bool last;
-    block_sum<A, NV>(v);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int i = 0; i < NV; ++i) partials[(size_t)i * nblk + blk] = (double)v[i];
-        __threadfence();
-        unsigned int t = atomicAdd(ticket, 1u);
-        last = (t == (unsigned int)nblk - 1);
-    }
-    __syncthreads();
-    if (!last) return false;
-    __threadfence();
-    sum_partials<NV>(partials, ticket, tot, nblk);
+    tot = sum_partials<NV>(partials, ticket, nblk);
     return true;
 }
 
@@ -215,11 +192,25 @@ __device__ __forceinline__ double block_total_t0(const float2 *partials, int n) 
     return total;
 }
 
-// Grid-wide sum over the launch's blocks (see grid_sum_of).
-template <typename A, int NV>
-__device__ __forceinline__ bool grid_sum(A (&v)[NV], double *partials, unsigned int *ticket,
-                                         double (&tot)[NV]) {
-    return grid_sum_of<A, NV>(v, partials, ticket, tot, (int)blockIdx.x, (int)gridDim.x);
+// Grid-wide sum of one value per thread over the launch's blocks.  Returns true
+// in exactly one of them (the last to finish), where thread 0 then holds the
+// FP64 total in tot.  partials: one double per block.
+template <typename A>
+__device__ __forceinline__ bool grid_sum(A v, double *partials, unsigned int *ticket,
+                                         double &tot) {
+    __shared__ bool last;
+    A s[1] = {v};
+    block_sum<A, 1>(s);
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = (double)s[0];
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    tot = sum_partials<1>(partials, ticket, (int)gridDim.x);
+    return true;
 }
 
 // Grid-wide sum of one value already reduced to thread 0 of each block of

@@ -262,12 +262,12 @@ k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__rest
             reinterpret_cast<float2 *>(partials)[blockIdx.x] = df_of((double)part[0]);
         return;
     }
-    double tot[1];
-    if (grid_sum<T, 1>(part, partials, &sc->ticket[0], tot) && threadIdx.x == 0) {
+    double tot;
+    if (grid_sum<T>(part[0], partials, &sc->ticket[0], tot) && threadIdx.x == 0) {
         if (sc->fault)
             sc->done = kFault;
         else
-            finalize(sc, fin, slot, tot[0]);
+            finalize(sc, fin, slot, tot);
     }
 }
 
@@ -526,12 +526,12 @@ k_spmv_lean(SpmvDev<float> A, const float *__restrict__ x, float *__restrict__ y
             reinterpret_cast<float2 *>(partials)[blockIdx.x] = df_of((double)part[0]);
         return;
     }
-    double tot[1];
-    if (grid_sum<float, 1>(part, partials, &sc->ticket[0], tot) && threadIdx.x == 0) {
+    double tot;
+    if (grid_sum<float>(part[0], partials, &sc->ticket[0], tot) && threadIdx.x == 0) {
         if (sc->fault)
             sc->done = kFault;
         else
-            finalize(sc, fin, slot, tot[0]);
+            finalize(sc, fin, slot, tot);
     }
 }
 
@@ -664,9 +664,9 @@ k_dot(const T *__restrict__ a, const T *__restrict__ b, long long n, double *par
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         part[0] = fma(a[i], b[i], part[0]);
-    double tot[1];
-    if (grid_sum<T, 1>(part, partials, &sc->ticket[1], tot) && threadIdx.x == 0)
-        finalize(sc, fin, slot, tot[0]);
+    double tot;
+    if (grid_sum<T>(part[0], partials, &sc->ticket[1], tot) && threadIdx.x == 0)
+        finalize(sc, fin, slot, tot);
 }
 
 template <typename T>

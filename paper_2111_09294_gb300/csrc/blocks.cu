@@ -105,45 +105,92 @@ void launch_scale_block_inverse(int n, const int *rowBlock, const int *bStart, c
 
 // y = M^-1 r block by block: unit u covers rows [unitRow0[u], unitRow1[u]) of
 // block unitBlk[u]; the CTA stages the block's whole r in shared memory (a
-// gather through idx), and each warp forms whole rows of the dense product
-// (lanes along the row, coalesced), summing in a fixed order.  The grid also
-// reduces r^T y into sc->ry (deterministic, last block).
+// gather through idx), and each warp forms four rows of the dense product at a
+// time (lanes along the rows, coalesced), each row summed in a fixed order.
+// The grid also reduces r^T y into sc->ry (deterministic, last block).
+//
+// Bound in FP32 by streaming the inverses (4 bytes per entry), in FP64 by the
+// FP64 units.  Four rows put 16 loads per lane in flight instead of four, the
+// first of them before the wait (the inverses are set-up data).  64 blocks of 540
+// to 1,740 dofs (24^3, FP32 solve): 3.96 ms before, 3.63 now.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 k_block_apply(BlkDev<T> B, const T *__restrict__ r, T *__restrict__ y, double *partials,
               Scalars *sc) {
+    constexpr int R = 4;
     __shared__ T rs[XDCG_MAX_BLOCK_DOFS];
-    pdl_wait();
-    if (sc->done != kRunning) return;
     const int u = blockIdx.x;
     const int b = B.unitBlk[u];
     const int p0 = B.bPos[b], nb = B.bPos[b + 1] - p0;
-    for (int j = threadIdx.x; j < nb; j += blockDim.x) rs[j] = r[B.idx[p0 + j]];
-    __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const T *Ab = B.A + B.aOff[b];
-    T part[1] = {T(0)};
-    for (int i = B.unitRow0[u] + warp; i < B.unitRow1[u]; i += kWarps) {
-        const T *row = Ab + (long long)i * nb;
-        T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
-        int j = lane;
-        for (; j + 96 < nb; j += 128) {
-            s0 = fma(__ldcs(row + j), rs[j], s0);
-            s1 = fma(__ldcs(row + j + 32), rs[j + 32], s1);
-            s2 = fma(__ldcs(row + j + 64), rs[j + 64], s2);
-            s3 = fma(__ldcs(row + j + 96), rs[j + 96], s3);
-        }
-        for (; j < nb; j += 32) s0 = fma(__ldcs(row + j), rs[j], s0);
-        T s = (s0 + s1) + (s2 + s3);
+    const int i1 = B.unitRow1[u];
+    T v[R][4];
+    // four entries of each of rows i, i + kWarps, ... (a row past the unit's end
+    // repeats its last one and is dropped)
+    auto load = [&](int i, int j) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            y[B.idx[p0 + i]] = s;
-            part[0] = fma(rs[i], s, part[0]);
+        for (int q = 0; q < R; ++q) {
+            const T *row = Ab + (long long)min(i + q * kWarps, i1 - 1) * nb;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) v[q][t] = __ldcs(row + j + 32 * t);
+        }
+    };
+    const int iFirst = B.unitRow0[u] + warp;
+    const bool early = __ldcg(&sc->done) == kRunning;   // may be stale: only loads depend on it
+    if (early && iFirst < i1 && lane + 96 < nb) load(iFirst, lane);
+    pdl_wait();
+    if (sc->done != kRunning) return;
+    for (int j = threadIdx.x; j < nb; j += blockDim.x) rs[j] = r[B.idx[p0 + j]];
+    __syncthreads();
+    T part = T(0);
+    for (int i = iFirst; i < i1; i += R * kWarps) {
+        T s[R][4] = {};
+        int j = lane;
+        bool have = early && i == iFirst;
+        for (; j + 96 < nb; j += 128) {
+            if (!have) load(i, j);
+            have = false;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const T x = rs[j + 32 * t];
+#pragma unroll
+                for (int q = 0; q < R; ++q) s[q][t] = fma(v[q][t], x, s[q][t]);
+            }
+        }
+        for (; j < nb; j += 32) {
+            T w[R];
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                w[q] = __ldcs(Ab + (long long)min(i + q * kWarps, i1 - 1) * nb + j);
+#pragma unroll
+            for (int q = 0; q < R; ++q) s[q][0] = fma(w[q], rs[j], s[q][0]);
+        }
+        // the rows' sums over the lanes by halving exchanges: lane 8 q gets row q
+        T a[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) a[q] = (s[q][0] + s[q][1]) + (s[q][2] + s[q][3]);
+#pragma unroll
+        for (int half = R / 2, o = 16; half > 0; half >>= 1, o >>= 1) {
+            const bool hi = (lane & o) != 0;
+#pragma unroll
+            for (int q = 0; q < half; ++q) {
+                const T send = hi ? a[q] : a[q + half], mine = hi ? a[q + half] : a[q];
+                a[q] = mine + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+        const int mineRow = i + (lane >> 3) * kWarps;
+        if ((lane & 7) == 0 && mineRow < i1) y[B.idx[p0 + mineRow]] = a[0];
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const T sum = __shfl_sync(0xffffffffu, a[0], 8 * q);
+            if (lane == 0 && i + q * kWarps < i1) part = fma(rs[i + q * kWarps], sum, part);
         }
     }
     double tot;
-    if (grid_sum<T>(part[0], partials, &sc->ticket[1], tot) && threadIdx.x == 0) sc->ry = tot;
+    if (grid_sum<T>(part, partials, &sc->ticket[1], tot) && threadIdx.x == 0) sc->ry = tot;
 }
 
 template <typename T>

@@ -409,7 +409,7 @@ struct PlainPath {
         launch_restrict(L.B, a, b, withW, c->g, zr, sc, st);
     }
     void coarse(const double *zr, int mode, Scalars *sc) {
-        launch_coarse(c->Einv, c->k, c->g, zr, c->nu, nullptr, mode, c->partials, sc, st);
+        launch_coarse(c->Einv, c->k, c->g, zr, c->nu, nullptr, mode, c->partials, nullptr, 0, sc, st);
     }
     void prolong(const double *y, double *p, int mode, Scalars *sc) {
         launch_prolong(L.B, c->nu, y, p, mode, sc, st);
@@ -559,11 +559,14 @@ __global__ void k_set_trigger(Scalars *sc, int mode, double delta2, double targe
 
 // nu = E^-1 g inside the FP32 iteration: the FP32 copy of E^-1 (default) or
 // the FP64 one (opt.coarse_fp64), both writing nu and its FP32 copy nu32
-void coarse_inner(xdcg_ctx *c, const double *zr, int mode, Scalars *sc, cudaStream_t st) {
+void coarse_inner(xdcg_ctx *c, const double *zr, int mode, Scalars *sc, cudaStream_t st,
+                  const double *rrPart = nullptr, int rrN = 0) {
     if (c->opt.coarse_fp64)
-        launch_coarse(c->Einv, c->k, c->g, zr, c->nu, c->nu32, mode, c->partials, sc, st);
+        launch_coarse(c->Einv, c->k, c->g, zr, c->nu, c->nu32, mode, c->partials, rrPart, rrN, sc,
+                      st);
     else
-        launch_coarse32(c->Einv32, c->k, c->g32, zr, c->nu, c->nu32, mode, c->partials, sc, st);
+        launch_coarse32(c->Einv32, c->k, c->g32, zr, c->nu, c->nu32, mode, c->partials, rrPart,
+                        rrN, sc, st);
 }
 
 // Algorithm 2 and the first direction: u~ = Z~ E^-1 Z~^T f~, r = f~ - K~ u~ (rA),
@@ -624,6 +627,8 @@ xdcg_status scaled_iterate(xdcg_ctx *c, float *u, float *rA, float *rB, float *p
         // product's end), past the region the restriction's own
         // reduction uses
         float2 *pqPart = reinterpret_cast<float2 *>(c->partials + kMaxGrid);
+        // and the restriction its units' sums of ||r||^2 for the coarse solve
+        double *rrPart = c->userBlocks ? nullptr : c->partials + 2 * kMaxGrid;
         if (m == 0) {
             launch_spmv<float>(L.A, p, q, nullptr, 0,
                                c->userBlocks ? c->partials : c->partials + kMaxGrid, sc,
@@ -638,11 +643,11 @@ xdcg_status scaled_iterate(xdcg_ctx *c, float *u, float *rA, float *rB, float *p
                                        c->partials, sc, s, c->y32);
                 c->launches += 2;
             } else {
-                launch_restrict_update_deferred(L.R, u, rc, rn, p, q, c->g, c->zr, c->partials, sc,
-                                                pqPart, L.A.grid, s);
+                launch_restrict_update_deferred(L.R, u, rc, rn, p, q, c->g, c->zr, rrPart, sc, pqPart,
+                                                L.A.grid, s);
             }
         } else if (m == 2) {
-            coarse_inner(c, c->zr, 2, sc, s);
+            coarse_inner(c, c->zr, 2, sc, s, rrPart, rrPart ? L.R.nUnits : 0);
         } else {
             launch_prolong_rows(L.R, c->nu32, c->userBlocks ? c->y32 : rn, p, 0, sc, s);
             c->launches += 4;
@@ -2999,7 +3004,8 @@ xdcg_status xdcg_precond(xdcg_ctx *c, const double *r, double *z) {
     CK(cudaMemcpyAsync(c->r64, r, c->n * sizeof(double), cudaMemcpyDeviceToDevice, st));
     PlainPath{c, c->L64, c->st}.update(nullptr, c->r64, nullptr, nullptr, c->y64, 1, c->aux);
     launch_restrict(c->L64.B, c->r64, c->y64, 1, c->g, c->zr, c->aux, st);
-    launch_coarse(c->Einv, c->k, c->g, c->zr, c->nu, nullptr, 0, c->partials, c->aux, st);
+    launch_coarse(c->Einv, c->k, c->g, c->zr, c->nu, nullptr, 0, c->partials, nullptr, 0, c->aux,
+                  st);
     launch_prolong(c->L64.B, c->nu, c->y64, z, 2, c->aux, st);
     c->launches += 4;
     CK(cudaStreamSynchronize(st));

@@ -616,7 +616,7 @@ __device__ __forceinline__ bool restrict_update_unit(const RowBoxDev &B, int uni
 // and block 0 records pq, alpha and counts the iteration (its += 1: the
 // launch's arguments do not depend on the iteration, so a captured batch of
 // iterations can be replayed), or the breakdown (or a failed wait of the
-// product).
+// product).  Its blocks' sums of ||r||^2 stay in partials, for the coarse solve.
 //
 // Bound by latency: 51 MB at 48^3, most of it from L2, between two grid-wide
 // dependencies.  48^3 (543 units): 28.8 us before (dependent loads after the
@@ -670,8 +670,14 @@ k_restrict_update(RowBoxDev B, float *u, const float *r_cur, float *r_next, cons
             : restrict_update_unit<6, YV, FEW>(B, unit, u, r_cur, r_next, p, q, yv, mode, g, zr,
                                                sc, stage, red, alpha_of, rr);
     if (!went || mode >= 2) return;
-    double tot;
-    if (grid_sum_t0<kRowThreads>((double)rr, partials, &sc->ticket[2], tot) && threadIdx.x == 0) {
+    if (deferred) {
+        if (threadIdx.x == 0) partials[blockIdx.x] = (double)rr;
+        return;
+    }
+    if (threadIdx.x == 0) partials[blockIdx.x] = (double)rr;
+    if (!last_block(&sc->ticket[2])) return;
+    const double tot = sum_slots<kRowThreads>(partials, (int)gridDim.x);
+    if (threadIdx.x == 0) {
         sc->rr = tot;
         sc->ry = tot;
         if (tot <= sc->tol2ff)
@@ -717,11 +723,11 @@ void launch_restrict_update(const RowBoxDev &B, float *u, const float *r_cur, fl
 
 void launch_restrict_update_deferred(const RowBoxDev &B, float *u, const float *r_cur,
                                      float *r_next, const float *p, const float *q, double *g,
-                                     double *zr, double *partials, Scalars *sc,
+                                     double *zr, double *rrPart, Scalars *sc,
                                      const float2 *pqPart, int pqN, cudaStream_t st) {
     auto launch = B.nUnits <= device_sm_count() ? launch_restrict_rows<false, true>
                                                 : launch_restrict_rows<false, false>;
-    launch(B, u, r_cur, r_next, p, q, nullptr, 0, g, zr, partials, sc, 1, pqPart, pqN, st);
+    launch(B, u, r_cur, r_next, p, q, nullptr, 0, g, zr, rrPart, sc, 1, pqPart, pqN, st);
 }
 
 // Triggers its dependent, the next product, only while its grid is small: the

@@ -175,22 +175,52 @@ void launch_symmetrize(double *E, int k, cudaStream_t st) {
 // ---- per-iteration coarse solve -------------------------------------------
 
 // Scalar updates shared by the coarse kernels (modes as for k_coarse); blk
-// holds the block's share of nu^T (Z^T r) in thread 0 (the few row sums
-// gathered through shared memory: no FP64 shuffle tree in every warp).
+// holds the share of nu^T (Z^T r) of row block rowBlk in thread 0 (the few row
+// sums gathered through shared memory: no FP64 shuffle tree in every warp).
+//
+// With rrPart the restriction left its rrN units' sums of ||r||^2 there, and the
+// launch has one more block, the first (rowBlk -1), which adds them while the
+// others stream E^-1; the last block to finish makes the restriction's stopping
+// tests (a stop leaves rho and beta as they are).  So the restriction needs no
+// reduction across its blocks (ticket, fences and FP64 trees): 18.5 -> 15.5 us at
+// 32^3, 16.3 -> 12.6 at 24^3, 26.5 -> 22.5 at 48^3.
 template <int THREADS>
-__device__ __forceinline__ void coarse_scalars(double blk, int mode, double *partials,
+__device__ __forceinline__ void coarse_scalars(double blk, int rowBlk, int mode,
+                                               double *partials, const double *rrPart, int rrN,
                                                Scalars *sc) {
-    double tot[1];
-    if (grid_sum_t0<THREADS>(blk, partials, &sc->ticket[3], tot[0]) && threadIdx.x == 0) {
-        if (mode == 1) {
-            sc->rho = sc->ry + tot[0];
-            sc->beta = 0.0;
-        } else if (mode >= 2) {
-            const double rho_new = sc->ry + tot[0];
-            const bool restart = mode == 3 && sc->rr > 4.0 * sc->scratch[3];
-            sc->beta = restart ? 0.0 : rho_new / sc->rho;
-            sc->rho = rho_new;
+    if (rowBlk < 0) {
+        const double rr = sum_slots<THREADS>(rrPart, rrN);
+        if (threadIdx.x == 0) {
+            sc->rr = rr;
+            sc->ry = rr;
         }
+        __syncthreads();
+    } else if (threadIdx.x == 0) {
+        partials[rowBlk] = blk;
+    }
+    if (!last_block(&sc->ticket[3])) return;
+    const double rr = __ldcg(&sc->rr), ry = __ldcg(&sc->ry), rho = sc->rho;
+    const double tol2ff = sc->tol2ff;
+    const int its = sc->its, max_it = sc->max_it;
+    const double tot = sum_slots<THREADS>(partials, (int)gridDim.x - (rrPart ? 1 : 0));
+    if (threadIdx.x != 0) return;
+    if (rrPart) {
+        const int stop = rr <= tol2ff ? kConverged
+                         : its >= max_it ? kMaxIter
+                         : !isfinite(rr) ? kBreakdown : kRunning;
+        if (stop != kRunning) {
+            sc->done = stop;
+            return;
+        }
+    }
+    if (mode == 1) {
+        sc->rho = ry + tot;
+        sc->beta = 0.0;
+    } else if (mode >= 2) {
+        const double rho_new = ry + tot;
+        const bool restart = mode == 3 && rr > 4.0 * sc->scratch[3];
+        sc->beta = restart ? 0.0 : rho_new / rho;
+        sc->rho = rho_new;
     }
 }
 
@@ -206,11 +236,12 @@ __device__ __forceinline__ void coarse_scalars(double blk, int mode, double *par
 __global__ void __launch_bounds__(kThreads)
 k_coarse(const double *__restrict__ Einv, int k, const double *__restrict__ g,
          const double *__restrict__ zr, double *nu, float *nu32, int mode, double *partials,
-         Scalars *sc) {
+         const double *rrPart, int rrN, Scalars *sc) {
     pdl_wait();
     if (sc->done != kRunning) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * kWarps + warp;
+    const int rowBlk = (int)blockIdx.x - (rrPart ? 1 : 0);
+    const int i = rowBlk < 0 ? k : rowBlk * kWarps + warp;
     double part[1] = {0.0};
     if (i < k) {
         const double *row = Einv + (size_t)i * k;
@@ -256,7 +287,7 @@ k_coarse(const double *__restrict__ Einv, int k, const double *__restrict__ g,
     double blk = 0.0;
     if (threadIdx.x == 0)
         for (int w = 0; w < kWarps; ++w) blk += rowPart[w];
-    coarse_scalars<kThreads>(blk, mode, partials, sc);
+    coarse_scalars<kThreads>(blk, rowBlk, mode, partials, rrPart, rrN, sc);
 }
 
 // nu = E^-1 g with E^-1 held in FP32, for the FP32 iteration of the mixed
@@ -282,14 +313,15 @@ template <int V>
 __global__ void __launch_bounds__(kCoarse32Threads)
 k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
            const double *__restrict__ zr, double *nu, float *nu32, int mode, double *partials,
-           Scalars *sc) {
+           const double *rrPart, int rrN, Scalars *sc) {
     constexpr int R = kCoarse32Rows, U = V == 4 ? 4 : 8;
     using E = typename std::conditional<V == 4, float4, float>::type;
     __shared__ float upper[R];
     const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i0 = blockIdx.x * R;
+    const int rowBlk = (int)blockIdx.x - (rrPart ? 1 : 0);
+    const int i0 = rowBlk < 0 ? k : rowBlk * R;
     const int nv = k / V, mid = (nv + 1) >> 1;
-    const int j0 = (h ? mid : 0) + lane, j1 = h ? nv : mid;
+    const int j0 = (h ? mid : 0) + lane, j1 = rowBlk < 0 ? 0 : (h ? nv : mid);
     const uint64_t keep = l2_keep_policy();
     const E *row[R];
 #pragma unroll
@@ -311,6 +343,10 @@ k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
     pdl_trigger();
     if (sc->done != kRunning) return;
     if (!early) load(j0);
+    // the row whose sum the lane will hold (one lane of eight)
+    const int r = lane >> 3, i = i0 + r;
+    const bool holder = (lane & 7) == 0;
+    const double zri = mode != 0 && h == 0 && holder && i < k ? zr[i] : 0.0;
     float s[R][4] = {};
     const E *gv = reinterpret_cast<const E *>(g32);
     for (int j = j0; j < j1; j += 32 * U) {
@@ -351,8 +387,6 @@ k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
     }
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-    const int r = lane >> 3, i = i0 + r;
-    const bool holder = (lane & 7) == 0;
     if (h == 1 && holder) upper[r] = v[0];
     __syncthreads();
     double blk = 0.0;
@@ -362,26 +396,28 @@ k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
             const float t = v[0] + upper[r];
             nu[i] = (double)t;
             nu32[i] = t;
-            if (mode != 0) part = (double)t * zr[i];
+            if (mode != 0) part = (double)t * zri;
         }
 #pragma unroll
         for (int q = 0; q < R; ++q) blk += __shfl_sync(0xffffffffu, part, 8 * q);
     }
-    coarse_scalars<kCoarse32Threads>(blk, mode, partials, sc);
+    coarse_scalars<kCoarse32Threads>(blk, rowBlk, mode, partials, rrPart, rrN, sc);
 }
 
 void launch_coarse32(const float *Einv, int k, const float *g32, const double *zr, double *nu,
-                     float *nu32, int mode, double *partials, Scalars *sc, cudaStream_t st) {
+                     float *nu32, int mode, double *partials, const double *rrPart, int rrN,
+                     Scalars *sc, cudaStream_t st) {
     const int grid = (k + kCoarse32Rows - 1) / kCoarse32Rows;
-    launch_pdl(k % 4 == 0 ? k_coarse32<4> : k_coarse32<1>, grid > 0 ? grid : 1, kCoarse32Threads,
-               0, st, Einv, k, g32, zr, nu, nu32, mode, partials, sc);
+    launch_pdl(k % 4 == 0 ? k_coarse32<4> : k_coarse32<1>, grid + (rrPart ? 1 : 0), kCoarse32Threads,
+               0, st, Einv, k, g32, zr, nu, nu32, mode, partials, rrPart, rrN, sc);
 }
 
 void launch_coarse(const double *Einv, int k, const double *g, const double *zr, double *nu,
-                   float *nu32, int mode, double *partials, Scalars *sc, cudaStream_t st) {
+                   float *nu32, int mode, double *partials, const double *rrPart, int rrN,
+                   Scalars *sc, cudaStream_t st) {
     const int grid = (k + kWarps - 1) / kWarps;
-    launch_pdl(k_coarse, grid > 0 ? grid : 1, kThreads, 0, st, Einv, k, g, zr, nu, nu32, mode,
-               partials, sc);
+    launch_pdl(k_coarse, grid + (rrPart ? 1 : 0), kThreads, 0, st, Einv, k, g, zr, nu, nu32, mode,
+               partials, rrPart, rrN, sc);
 }
 
 }  // namespace xdcg

@@ -262,19 +262,23 @@ void launch_prolong_rows(const RowBoxDev &B, const float *nu32, const float *y, 
                          int mode, Scalars *sc, cudaStream_t st);
 // The FP32 iteration's restriction (mode 0) after a product launched with
 // kFinDefer: it adds the product's block sums of p^T q (pqPart, pqN of them)
-// itself, takes alpha from them and counts the iteration in sc->its.
+// itself, takes alpha from them and counts the iteration in sc->its; its units'
+// sums of ||r||^2 go to rrPart for the coarse solve to add and test.
 void launch_restrict_update_deferred(const RowBoxDev &B, float *u, const float *r_cur,
                                      float *r_next, const float *p, const float *q, double *g,
-                                     double *zr, double *partials, Scalars *sc,
+                                     double *zr, double *rrPart, Scalars *sc,
                                      const float2 *pqPart, int pqN, cudaStream_t st);
 void launch_to_colmajor(int nItems, const int *itemBox, const int *rowStart,
                         const unsigned char *itemB, const long long *srcOff,
                         const int *boxRowPtr, const long long *boxBase, const int *menr,
                         const float *src, float *dst, cudaStream_t st);
 
-// nu = E^-1 g (FP64; nu32 optional FP32 copy)
+// nu = E^-1 g (FP64; nu32 optional FP32 copy).  rrPart (may be null): the rrN
+// sums of ||r||^2 that a restriction launched with launch_restrict_update_deferred
+// left for the coarse solve to add and test.
 void launch_coarse(const double *Einv, int k, const double *g, const double *zr, double *nu,
-                   float *nu32, int mode, double *partials, Scalars *sc, cudaStream_t st);
+                   float *nu32, int mode, double *partials, const double *rrPart, int rrN,
+                   Scalars *sc, cudaStream_t st);
 
 template <typename T>
 void launch_dot(const T *a, const T *b, long long n, double *partials, Scalars *sc, int fin,
@@ -405,7 +409,8 @@ void launch_build_E(int nSeg, const int *segBox, const int *segOwner, const int 
                     const ZvalDev &Zv, int k, double *E, cudaStream_t st);
 void launch_symmetrize(double *E, int k, cudaStream_t st);
 void launch_coarse32(const float *Einv, int k, const float *g32, const double *zr, double *nu,
-                     float *nu32, int mode, double *partials, Scalars *sc, cudaStream_t st);
+                     float *nu32, int mode, double *partials, const double *rrPart, int rrN,
+                     Scalars *sc, cudaStream_t st);
 void launch_cast_f32(const double *a, float *b, long long n, cudaStream_t st);
 void launch_scale_blocks(const KinDev &K, const int *blockRow, long long nnzb, const FacDev &F,
                          double *Kt, cudaStream_t st);

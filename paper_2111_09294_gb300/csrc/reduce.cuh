@@ -213,61 +213,61 @@ __device__ __forceinline__ bool grid_sum(A v, double *partials, unsigned int *ti
     return true;
 }
 
-// Grid-wide sum of one value already reduced to thread 0 of each block of
-// THREADS threads: returns true in the last block to finish, where thread 0
-// holds the FP64 total.  The order of the sum is that of 256 threads whatever
-// THREADS: slot t = 0 .. 255 adds partials t, t + 256, ..., then the tree over
-// the 32 slots of a warp and the tree over the eight warps; a thread of a
-// smaller block takes 256 / THREADS slots.
+// Sum of n block partials by one block of THREADS threads, valid in thread 0.
+// The order of the sum is that of 256 threads whatever THREADS: slot t = 0 ..
+// 255 adds partials t, t + 256, ..., then the tree over the 32 slots of a warp and
+// the tree over the eight warps; a thread of a smaller block takes 256 / THREADS
+// slots.
 template <int THREADS>
-__device__ __forceinline__ bool grid_sum_t0(double v, double *partials, unsigned int *ticket,
-                                            double &tot) {
+__device__ __forceinline__ double sum_slots(const double *p, int n) {
     constexpr int Q = kThreads / THREADS;
     static_assert(Q == 1 || Q == 4, "");
-    __shared__ bool last;
     __shared__ double sums[kWarps];
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = v;
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return false;
-    __threadfence();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = (int)gridDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double s[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) s[q] = 0.0;
     for (int b = threadIdx.x; b < n; b += kThreads)
 #pragma unroll
         for (int q = 0; q < Q; ++q)
-            if (b + q * THREADS < n) s[q] += __ldcg(partials + b + q * THREADS);
+            if (b + q * THREADS < n) s[q] += __ldcg(p + b + q * THREADS);
     int o = 16;
     if (Q == 4) {   // halving exchanges: lanes 8 q .. 8 q + 7 keep the sums of slot set q
 #pragma unroll
         for (int half = 2; half > 0; half >>= 1, o >>= 1) {
             const bool hi = (lane & o) != 0;
 #pragma unroll
-            for (int i = 0; i < half; ++i) {
-                const double send = hi ? s[i] : s[(i + half) % Q];
-                const double mine = hi ? s[(i + half) % Q] : s[i];
-                s[i] = mine + __shfl_xor_sync(0xffffffffu, send, o);
+            for (int j = 0; j < half; ++j) {
+                const double send = hi ? s[j] : s[(j + half) % Q];
+                const double mine = hi ? s[(j + half) % Q] : s[j];
+                s[j] = mine + __shfl_xor_sync(0xffffffffu, send, o);
             }
         }
     }
     for (; o > 0; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
     if (lane % (32 / Q) == 0) sums[warp + (THREADS / 32) * (lane / (32 / Q))] = s[0];
     __syncthreads();
+    double t = 0.0;
     if (warp == 0) {
-        double t = lane < kWarps ? sums[lane] : 0.0;
+        t = lane < kWarps ? sums[lane] : 0.0;
 #pragma unroll
-        for (int p = 4; p > 0; p >>= 1) t += __shfl_xor_sync(0xffffffffu, t, p);
-        if (lane == 0) {
-            tot = t;
-            *ticket = 0u;
-        }
+        for (int l = 4; l > 0; l >>= 1) t += __shfl_xor_sync(0xffffffffu, t, l);
     }
-    return true;
+    return t;
+}
+
+// True in the last block of the launch to get here, which may read what thread 0
+// of every block wrote before.
+__device__ __forceinline__ bool last_block(unsigned int *ticket) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (last) *ticket = 0u;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
 }
 
 // Reports the run's state to the host (one thread of a kernel that ends an

@@ -104,6 +104,7 @@ struct xdcg_ctx {
     double *g = nullptr, *zr = nullptr, *nu = nullptr;
     float *nu32 = nullptr;
     double *partials = nullptr;
+    double *updPart = nullptr;     // the FP64 update's block sums
     Scalars *sc = nullptr, *sc32 = nullptr, *aux = nullptr;
     Scalars *h_sc = nullptr;   // pinned
     Progress *h_prog = nullptr; // pinned: what the running solve reports per iteration
@@ -402,14 +403,20 @@ struct PlainPath {
             launch_block_apply<double>(L.J, r, y, c->partials, sc, st);
             c->launches++;
         } else {
-            launch_update(L.N, u, r, p, q, y, mode, c->partials, sc, st);
+            launch_update(L.N, u, r, p, q, y, mode, c->updPart, sc, st);
         }
     }
     void restrict_(const double *a, const double *b, int withW, double *zr, Scalars *sc) {
         launch_restrict(L.B, a, b, withW, c->g, zr, sc, st);
     }
+    // an iteration's (or the start's) coarse solve adds the update's sums
+    ResidualSums sums(int mode) const {
+        if (mode == 0 || c->userBlocks) return ResidualSums{nullptr, 0, 0};
+        return ResidualSums{c->updPart, update_units(L.N), 2};
+    }
     void coarse(const double *zr, int mode, Scalars *sc) {
-        launch_coarse(c->Einv, c->k, c->g, zr, c->nu, nullptr, mode, c->partials, nullptr, 0, sc, st);
+        launch_coarse(c->Einv, c->k, c->g, zr, c->nu, nullptr, mode, c->partials,
+                      sums(mode), sc, st);
     }
     void prolong(const double *y, double *p, int mode, Scalars *sc) {
         launch_prolong(L.B, c->nu, y, p, mode, sc, st);
@@ -560,13 +567,12 @@ __global__ void k_set_trigger(Scalars *sc, int mode, double delta2, double targe
 // nu = E^-1 g inside the FP32 iteration: the FP32 copy of E^-1 (default) or
 // the FP64 one (opt.coarse_fp64), both writing nu and its FP32 copy nu32
 void coarse_inner(xdcg_ctx *c, const double *zr, int mode, Scalars *sc, cudaStream_t st,
-                  const double *rrPart = nullptr, int rrN = 0) {
+                  ResidualSums sums = ResidualSums{nullptr, 0, 0}) {
     if (c->opt.coarse_fp64)
-        launch_coarse(c->Einv, c->k, c->g, zr, c->nu, c->nu32, mode, c->partials, rrPart, rrN, sc,
-                      st);
+        launch_coarse(c->Einv, c->k, c->g, zr, c->nu, c->nu32, mode, c->partials, sums, sc, st);
     else
-        launch_coarse32(c->Einv32, c->k, c->g32, zr, c->nu, c->nu32, mode, c->partials, rrPart,
-                        rrN, sc, st);
+        launch_coarse32(c->Einv32, c->k, c->g32, zr, c->nu, c->nu32, mode, c->partials, sums, sc,
+                        st);
 }
 
 // Algorithm 2 and the first direction: u~ = Z~ E^-1 Z~^T f~, r = f~ - K~ u~ (rA),
@@ -647,7 +653,7 @@ xdcg_status scaled_iterate(xdcg_ctx *c, float *u, float *rA, float *rB, float *p
                                                 L.A.grid, s);
             }
         } else if (m == 2) {
-            coarse_inner(c, c->zr, 2, sc, s, rrPart, rrPart ? L.R.nUnits : 0);
+            coarse_inner(c, c->zr, 2, sc, s, ResidualSums{rrPart, L.R.nUnits, 1});
         } else {
             launch_prolong_rows(L.R, c->nu32, c->userBlocks ? c->y32 : rn, p, 0, sc, s);
             c->launches += 4;
@@ -2522,6 +2528,7 @@ xdcg_status setup_impl(xdcg_ctx *c, const xdcg_matrix *K, const xdcg_deflation *
     c->g = dalloc<double>(c, k); c->zr = dalloc<double>(c, k); c->nu = dalloc<double>(c, k);
     c->nu32 = dalloc<float>(c, k);
     c->partials = dalloc<double>(c, 4 * (size_t)kMaxGrid);
+    c->updPart = dalloc<double>(c, 2 * (size_t)update_units(c->L64.N));
     c->sc = dalloc<Scalars>(c, 1); c->sc32 = dalloc<Scalars>(c, 1); c->aux = dalloc<Scalars>(c, 1);
     if (c->opt.record_history) {
         c->hist = dalloc<double>(c, (size_t)c->opt.max_iter + 1);
@@ -2551,7 +2558,7 @@ xdcg_status setup_impl(xdcg_ctx *c, const xdcg_matrix *K, const xdcg_deflation *
         if (!spmm_prepare()) return XDCG_CUDA_ERROR;
     }
     if (!c->u64 || !c->r64 || !c->p64 || !c->q64 || !c->y64 || !c->f64 || !c->uh64 || !c->g ||
-        !c->zr || !c->nu || !c->nu32 || !c->partials || !c->sc || !c->sc32 || !c->aux)
+        !c->zr || !c->nu || !c->nu32 || !c->partials || !c->updPart || !c->sc || !c->sc32 || !c->aux)
         return XDCG_OOM;
     CK(cudaMemsetAsync(c->sc, 0, sizeof(Scalars), st));
     CK(cudaMemsetAsync(c->sc32, 0, sizeof(Scalars), st));
@@ -3004,8 +3011,8 @@ xdcg_status xdcg_precond(xdcg_ctx *c, const double *r, double *z) {
     CK(cudaMemcpyAsync(c->r64, r, c->n * sizeof(double), cudaMemcpyDeviceToDevice, st));
     PlainPath{c, c->L64, c->st}.update(nullptr, c->r64, nullptr, nullptr, c->y64, 1, c->aux);
     launch_restrict(c->L64.B, c->r64, c->y64, 1, c->g, c->zr, c->aux, st);
-    launch_coarse(c->Einv, c->k, c->g, c->zr, c->nu, nullptr, 0, c->partials, nullptr, 0, c->aux,
-                  st);
+    launch_coarse(c->Einv, c->k, c->g, c->zr, c->nu, nullptr, 0, c->partials,
+                  ResidualSums{nullptr, 0, 0}, c->aux, st);
     launch_prolong(c->L64.B, c->nu, c->y64, z, 2, c->aux, st);
     c->launches += 4;
     CK(cudaStreamSynchronize(st));

@@ -178,21 +178,29 @@ void launch_symmetrize(double *E, int k, cudaStream_t st) {
 // holds the share of nu^T (Z^T r) of row block rowBlk in thread 0 (the few row
 // sums gathered through shared memory: no FP64 shuffle tree in every warp).
 //
-// With rrPart the restriction left its rrN units' sums of ||r||^2 there, and the
-// launch has one more block, the first (rowBlk -1), which adds them while the
-// others stream E^-1; the last block to finish makes the restriction's stopping
-// tests (a stop leaves rho and beta as they are).  So the restriction needs no
-// reduction across its blocks (ticket, fences and FP64 trees): 18.5 -> 15.5 us at
-// 32^3, 16.3 -> 12.6 at 24^3, 26.5 -> 22.5 at 48^3.
+// With sums.part the kernel before left its blocks' sums there (ResidualSums: the
+// FP32 restriction those of ||r||^2, the FP64 update those of ||r||^2 and r^T y),
+// and the launch has one more block, the first (rowBlk -1), which adds them while
+// the others stream E^-1; the last block to finish makes the stopping tests (a
+// stop leaves rho and beta as they are).  So those kernels need no reduction
+// across their blocks (ticket, fences and FP64 trees): FP32 restriction 18.5 ->
+// 15.5 us at 32^3, 16.3 -> 12.6 at 24^3, 26.5 -> 22.5 at 48^3; FP64 update 16.3 -> 13.7 at
+// 8^3, 17.1 -> 14.4 at 24^3.
 template <int THREADS>
 __device__ __forceinline__ void coarse_scalars(double blk, int rowBlk, int mode,
-                                               double *partials, const double *rrPart, int rrN,
+                                               double *partials, const ResidualSums &sums,
                                                Scalars *sc) {
     if (rowBlk < 0) {
-        const double rr = sum_slots<THREADS>(rrPart, rrN);
-        if (threadIdx.x == 0) {
-            sc->rr = rr;
-            sc->ry = rr;
+        if (sums.values == 2) {
+            const double t = sum_partials<2>(sums.part, &sc->ticket[2], sums.n);
+            if (threadIdx.x == 0) sc->rr = t;
+            if (threadIdx.x == 1) sc->ry = t;
+        } else {
+            const double rr = sum_slots<THREADS>(sums.part, sums.n);
+            if (threadIdx.x == 0) {
+                sc->rr = rr;
+                sc->ry = rr;
+            }
         }
         __syncthreads();
     } else if (threadIdx.x == 0) {
@@ -202,12 +210,13 @@ __device__ __forceinline__ void coarse_scalars(double blk, int rowBlk, int mode,
     const double rr = __ldcg(&sc->rr), ry = __ldcg(&sc->ry), rho = sc->rho;
     const double tol2ff = sc->tol2ff;
     const int its = sc->its, max_it = sc->max_it;
-    const double tot = sum_slots<THREADS>(partials, (int)gridDim.x - (rrPart ? 1 : 0));
+    const double tot = sum_slots<THREADS>(partials, (int)gridDim.x - (sums.part ? 1 : 0));
     if (threadIdx.x != 0) return;
-    if (rrPart) {
+    if (sums.part) {
+        if (sc->hist && its < sc->histCap) sc->hist[its] = rr;
         const int stop = rr <= tol2ff ? kConverged
                          : its >= max_it ? kMaxIter
-                         : !isfinite(rr) ? kBreakdown : kRunning;
+                         : !isfinite(rr) || !isfinite(ry) ? kBreakdown : kRunning;
         if (stop != kRunning) {
             sc->done = stop;
             return;
@@ -236,11 +245,11 @@ __device__ __forceinline__ void coarse_scalars(double blk, int rowBlk, int mode,
 __global__ void __launch_bounds__(kThreads)
 k_coarse(const double *__restrict__ Einv, int k, const double *__restrict__ g,
          const double *__restrict__ zr, double *nu, float *nu32, int mode, double *partials,
-         const double *rrPart, int rrN, Scalars *sc) {
+         ResidualSums sums, Scalars *sc) {
     pdl_wait();
     if (sc->done != kRunning) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rowBlk = (int)blockIdx.x - (rrPart ? 1 : 0);
+    const int rowBlk = (int)blockIdx.x - (sums.part ? 1 : 0);
     const int i = rowBlk < 0 ? k : rowBlk * kWarps + warp;
     double part[1] = {0.0};
     if (i < k) {
@@ -287,7 +296,7 @@ k_coarse(const double *__restrict__ Einv, int k, const double *__restrict__ g,
     double blk = 0.0;
     if (threadIdx.x == 0)
         for (int w = 0; w < kWarps; ++w) blk += rowPart[w];
-    coarse_scalars<kThreads>(blk, rowBlk, mode, partials, rrPart, rrN, sc);
+    coarse_scalars<kThreads>(blk, rowBlk, mode, partials, sums, sc);
 }
 
 // nu = E^-1 g with E^-1 held in FP32, for the FP32 iteration of the mixed
@@ -313,12 +322,12 @@ template <int V>
 __global__ void __launch_bounds__(kCoarse32Threads)
 k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
            const double *__restrict__ zr, double *nu, float *nu32, int mode, double *partials,
-           const double *rrPart, int rrN, Scalars *sc) {
+           ResidualSums sums, Scalars *sc) {
     constexpr int R = kCoarse32Rows, U = V == 4 ? 4 : 8;
     using E = typename std::conditional<V == 4, float4, float>::type;
     __shared__ float upper[R];
     const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rowBlk = (int)blockIdx.x - (rrPart ? 1 : 0);
+    const int rowBlk = (int)blockIdx.x - (sums.part ? 1 : 0);
     const int i0 = rowBlk < 0 ? k : rowBlk * R;
     const int nv = k / V, mid = (nv + 1) >> 1;
     const int j0 = (h ? mid : 0) + lane, j1 = rowBlk < 0 ? 0 : (h ? nv : mid);
@@ -401,23 +410,23 @@ k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
 #pragma unroll
         for (int q = 0; q < R; ++q) blk += __shfl_sync(0xffffffffu, part, 8 * q);
     }
-    coarse_scalars<kCoarse32Threads>(blk, rowBlk, mode, partials, rrPart, rrN, sc);
+    coarse_scalars<kCoarse32Threads>(blk, rowBlk, mode, partials, sums, sc);
 }
 
 void launch_coarse32(const float *Einv, int k, const float *g32, const double *zr, double *nu,
-                     float *nu32, int mode, double *partials, const double *rrPart, int rrN,
+                     float *nu32, int mode, double *partials, ResidualSums sums,
                      Scalars *sc, cudaStream_t st) {
     const int grid = (k + kCoarse32Rows - 1) / kCoarse32Rows;
-    launch_pdl(k % 4 == 0 ? k_coarse32<4> : k_coarse32<1>, grid + (rrPart ? 1 : 0), kCoarse32Threads,
-               0, st, Einv, k, g32, zr, nu, nu32, mode, partials, rrPart, rrN, sc);
+    launch_pdl(k % 4 == 0 ? k_coarse32<4> : k_coarse32<1>, grid + (sums.part ? 1 : 0), kCoarse32Threads,
+               0, st, Einv, k, g32, zr, nu, nu32, mode, partials, sums, sc);
 }
 
 void launch_coarse(const double *Einv, int k, const double *g, const double *zr, double *nu,
-                   float *nu32, int mode, double *partials, const double *rrPart, int rrN,
+                   float *nu32, int mode, double *partials, ResidualSums sums,
                    Scalars *sc, cudaStream_t st) {
     const int grid = (k + kWarps - 1) / kWarps;
-    launch_pdl(k_coarse, grid + (rrPart ? 1 : 0), kThreads, 0, st, Einv, k, g, zr, nu, nu32, mode,
-               partials, rrPart, rrN, sc);
+    launch_pdl(k_coarse, grid + (sums.part ? 1 : 0), kThreads, 0, st, Einv, k, g, zr, nu, nu32, mode,
+               partials, sums, sc);
 }
 
 }  // namespace xdcg

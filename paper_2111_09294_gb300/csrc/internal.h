@@ -206,9 +206,12 @@ int spmv_persistent_grid(int nSlicesTotal, int shape);
 template <typename T>
 int spmv_shape_count();
 
+// block sums of ||r||^2 and r^T y to part (2 * update_units(N) doubles), for the
+// coarse solve
 void launch_update(const NodeDev<double> &N, double *u, double *r, const double *p,
-                   const double *q, double *y, int mode, double *partials, Scalars *sc,
+                   const double *q, double *y, int mode, double *part, Scalars *sc,
                    cudaStream_t st);
+int update_units(const NodeDev<double> &N);
 
 // Row-parallel form of the block-scaled FP32 path: per box, the rows of its
 // own nodes (Z~, column-major: column c of box s at Z + zBase[s] + c * R_s;
@@ -273,11 +276,17 @@ void launch_to_colmajor(int nItems, const int *itemBox, const int *rowStart,
                         const int *boxRowPtr, const long long *boxBase, const int *menr,
                         const float *src, float *dst, cudaStream_t st);
 
-// nu = E^-1 g (FP64; nu32 optional FP32 copy).  rrPart (may be null): the rrN
-// sums of ||r||^2 that a restriction launched with launch_restrict_update_deferred
-// left for the coarse solve to add and test.
+// Block sums that the coarse solve adds beside its own work, making the stopping
+// tests on them: values = 1, ||r||^2 (n of them, launch_restrict_update_deferred);
+// values = 2, ||r||^2 and then r^T y (n of each, launch_update).
+struct ResidualSums {
+    const double *part;   // null: the scalars are set already
+    int n, values;
+};
+
+// nu = E^-1 g (FP64; nu32 optional FP32 copy)
 void launch_coarse(const double *Einv, int k, const double *g, const double *zr, double *nu,
-                   float *nu32, int mode, double *partials, const double *rrPart, int rrN,
+                   float *nu32, int mode, double *partials, ResidualSums sums,
                    Scalars *sc, cudaStream_t st);
 
 template <typename T>
@@ -409,7 +418,7 @@ void launch_build_E(int nSeg, const int *segBox, const int *segOwner, const int 
                     const ZvalDev &Zv, int k, double *E, cudaStream_t st);
 void launch_symmetrize(double *E, int k, cudaStream_t st);
 void launch_coarse32(const float *Einv, int k, const float *g32, const double *zr, double *nu,
-                     float *nu32, int mode, double *partials, const double *rrPart, int rrN,
+                     float *nu32, int mode, double *partials, ResidualSums sums,
                      Scalars *sc, cudaStream_t st);
 void launch_cast_f32(const double *a, float *b, long long n, cudaStream_t st);
 void launch_scale_blocks(const KinDev &K, const int *blockRow, long long nnzb, const FacDev &F,

@@ -116,16 +116,17 @@ __device__ __forceinline__ void update_tip_half(const double (&Lr)[15], const do
 // per half-warp).  Each unit's two sums are the tree over its lanes and then
 // its 8 warps (or nodes); the two values share the shuffles and FP64 adds of
 // a tree (they are exchanged at its first step, one half-warp keeping each),
-// because FP64 instructions are what these trees cost.
+// because FP64 instructions are what these trees cost.  The units' sums are
+// added by the coarse solve (ResidualSums).
 //
 // Bound by FP64 issue and memory latency: everything that set-up fixed (node
 // lists, factors) is loaded before the wait for the product, everything else
 // in one round trip after it.  48^3 (373k dofs, 115k nodes, 1,932 of them with
-// 15 dofs): 44.9 us before, 28.3 now; 8.9k dofs: 17.4 before, 16.7 now
+// 15 dofs): 44.9 us before, 24.4 now; 8.9k dofs: 17.4 before, 14.2 now
 // (event-timed in the solve, as all figures of this kernel).
 __global__ void __launch_bounds__(kThreads, 3)
 k_update(NodeDev<double> N, double *u, double *r, const double *p, const double *q, double *y,
-         int mode, int nb3, int nb6, int nUnits, double *partials, Scalars *sc) {
+         int mode, int nb3, int nb6, int nUnits, double *part, const Scalars *sc) {
     // the 15-dof nodes' blocks, whose substitutions take longest, are
     // scheduled first; their units come last in the sums
     const int nb15 = (int)gridDim.x - nb3 - nb6;
@@ -191,7 +192,6 @@ k_update(NodeDev<double> N, double *u, double *r, const double *p, const double 
         for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if ((lane & 7) == 0) sums[(lane >> 3) & 1][hw] = s;
     }
-    __shared__ bool last;
     __syncthreads();
     if (warp == 0) {
         // lane = 16 (unit of the block) + 8 (value) + warp or node of the unit
@@ -200,41 +200,24 @@ k_update(NodeDev<double> N, double *u, double *r, const double *p, const double 
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         const int unit = tips ? nb3 + nb6 + 2 * (bid - nb3 - nb6) + un : bid;
-        if ((lane & 7) == 0 && (un == 0 || tips) && unit < nUnits) {
-            partials[(size_t)val * nUnits + unit] = s;
-            __threadfence();
-        }
-        __syncwarp();
-        if (lane == 0) last = atomicAdd(&sc->ticket[2], 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    const double sum = sum_partials<2>(partials, &sc->ticket[2], nUnits);
-    if (warp != 0) return;
-    const double tot[2] = {sum, __shfl_sync(0xffffffffu, sum, 1)};
-    if (threadIdx.x == 0) {
-        sc->ry = tot[1];
-        sc->rr = tot[0];
-        if (sc->hist && sc->its < sc->histCap) sc->hist[sc->its] = tot[0];
-        if (tot[0] <= sc->tol2ff)
-            sc->done = kConverged;
-        else if (sc->its >= sc->max_it)
-            sc->done = kMaxIter;
-        else if (!isfinite(tot[0]) || !isfinite(tot[1]))
-            sc->done = kBreakdown;
+        if ((lane & 7) == 0 && (un == 0 || tips) && unit < nUnits)
+            part[(size_t)val * nUnits + unit] = s;
     }
 }
 
 static inline int cdiv(long long a, int b) { return (int)((a + b - 1) / b); }
 
+int update_units(const NodeDev<double> &N) {
+    return std::max(cdiv(N.nStd, kThreads) + cdiv(N.nH, kThreads) + cdiv(N.nT, kWarps), 1);
+}
+
 void launch_update(const NodeDev<double> &N, double *u, double *r, const double *p,
-                   const double *q, double *y, int mode, double *partials, Scalars *sc,
+                   const double *q, double *y, int mode, double *part, Scalars *sc,
                    cudaStream_t st) {
     const int nb3 = cdiv(N.nStd, kThreads), nb6 = cdiv(N.nH, kThreads), nu15 = cdiv(N.nT, kWarps);
     const int grid = std::max(nb3 + nb6 + (nu15 + 1) / 2, 1);
-    launch_pdl(k_update, grid, kThreads, 0, st, N, u, r, p, q, y, mode, nb3, nb6,
-               std::max(nb3 + nb6 + nu15, 1), partials, sc);
+    launch_pdl(k_update, grid, kThreads, 0, st, N, u, r, p, q, y, mode, nb3, nb6, update_units(N),
+               part, (const Scalars *)sc);
 }
 
 // ---- set-up: node-block Cholesky (FP64) ------------------------------------

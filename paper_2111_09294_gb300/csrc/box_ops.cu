@@ -36,13 +36,15 @@ namespace xdcg {
 //
 // 48^3 (512 boxes, 373k dofs): 82.9 us before (one CTA of 128 threads per box,
 // one warp set doing both sums, loads exposed per four nodes, a six-way
-// divergent switch per node), 57.3 now; 24^3 (64 boxes): 56.6 before, 30.4
-// now; 12^3 (8 boxes): 61.9 before, 32.3 now.
+// divergent switch per node), 47.8 now; 24^3 (64 boxes): 56.6 before, 28.8 now;
+// 12^3 (8 boxes): 61.9 before, 30.9 now.  Two CTAs per SM: with three the longest
+// chains share their SM's FP64 units with more of the others (57.5 us at 48^3),
+// with one the gathers are exposed (58.9).
 
 constexpr int kBoxThreads = 256;
 constexpr int kExtChunk = 880, kOwnChunk = 240;   // records / nodes per chunk: multiples of 20, 8
 constexpr int kOwnRecChunk = 560;                 // records of Z by value (the same memory)
-constexpr int kAhead = 6;                         // groups of W in flight per lane
+constexpr int kAhead = 12;                         // groups of W in flight per lane
 
 struct OwnGeo {
     double a[kOwnChunk * 6], x[kOwnChunk * 3];
@@ -106,7 +108,7 @@ __device__ __forceinline__ double rigid_col(int c, const double *a, const double
 }
 
 template <bool EXPL>
-__global__ void __launch_bounds__(kBoxThreads, 3)
+__global__ void __launch_bounds__(kBoxThreads, 2)
 k_restrict(BoxDev<double> B, const double *a, const double *b, int withW, double *g, double *zr,
            const Scalars *sc) {
     __shared__ double sv[kExtChunk * 3];

@@ -1036,13 +1036,7 @@ void batch_replace(BatchRun &R, unsigned M, cudaStream_t st) {
     launch_batch_open(c->bs, c->bSlots, M, st);
     launch_bwd_accum_b<MB>(c->nNodes, m, L.dofStart64, L.dofStart32, L.F, c->bU32, c->bs, R.U, n,
                            st);
-    int nr = 0;
-    for (int j = 0; j < m; ++j)
-        if ((M >> j) & 1u) {
-            launch_spmv<double>(c->L64.A, R.U + j * n, c->bR64 + j * n, R.F + j * n, 1,
-                                c->partials, c->bSlots + j, kFinStore, 0, st);
-            ++nr;
-        }
+    launch_residuals(c->L64.A, R.U, c->bR64, R.F, n, M, c->partials, c->bSlots, st);
     launch_batch_judge(c->bs, c->bSlots, m, st);
     launch_fwd_scale_b<MB>(c->nNodes, m, L.dofStart64, L.dofStart32, L.F, c->bR64, n, c->bs,
                            c->bRA, c->bRB, st);
@@ -1050,7 +1044,7 @@ void batch_replace(BatchRun &R, unsigned M, cudaStream_t st) {
     launch_coarse_b<MB>(coarse_args(c, m, 3), st);
     launch_prolong_b<MB>(prolong_args(c, m, 3), st);
     launch_batch_arm(c->bs, m, 0, st);
-    c->launches += 8 + nr;
+    c->launches += 9;
 }
 
 // per-column results from the final scalars; the system's status

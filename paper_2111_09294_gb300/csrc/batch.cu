@@ -1143,25 +1143,30 @@ __global__ void k_fwd_scale_b(int nNodes, int m, const int *nat, const int *ot, 
 template <int MB>
 __global__ void k_bwd_accum_b(int nNodes, int m, const int *nat, const int *in, FacDev F,
                               float *ut, const BatchScalars *bs, double *u, long long ldu) {
+    // one division per column and block, not one per thread (FP64)
+    __shared__ double inv[MB];
+    if (threadIdx.x < MB) inv[threadIdx.x] = 1.0 / bs->scale[threadIdx.x];
+    __syncthreads();
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (t >= (long long)nNodes * MB) return;
     const int I = (int)(t / MB), j = (int)(t % MB);
     if (j >= m || !bs->repl[j]) return;
     const int b = nat[I + 1] - nat[I], d0 = in[I], o0 = nat[I];
-    const double inv = 1.0 / bs->scale[j];
     const int q = F.nodeIdx[I];
     with_node_size(b, [&](auto Bc) {
         constexpr int B = decltype(Bc)::value;
-        double x[B];
+        double x[B], uv[B];
 #pragma unroll
         for (int i = 0; i < B; ++i) {
-            float *e = ut + (size_t)(d0 + i) * MB + j;
-            x[i] = (double)*e;
-            *e = 0.0f;
+            x[i] = (double)ut[(size_t)(d0 + i) * MB + j];
+            uv[i] = u[j * ldu + o0 + i];
         }
         bwd_solve_fixed<B>(F, q, x);
 #pragma unroll
-        for (int i = 0; i < B; ++i) u[j * ldu + o0 + i] += inv * x[i];
+        for (int i = 0; i < B; ++i) {
+            ut[(size_t)(d0 + i) * MB + j] = 0.0f;
+            u[j * ldu + o0 + i] = uv[i] + inv[j] * x[i];
+        }
     });
 }
 

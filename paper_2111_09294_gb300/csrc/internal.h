@@ -199,6 +199,15 @@ int device_sm_count();
 template <typename T>
 void launch_spmv(const SpmvDev<T> &A, const T *x, T *y, const T *b, int residual_mode,
                  double *partials, Scalars *sc, int fin, int slot, cudaStream_t st);
+// the columns of a launch over several (launch_residuals): four bits each, the
+// column + 1, in order; 0: one column, the pointers as given
+struct SpmvCols {
+    unsigned long long list;
+    long long ld;
+};
+void launch_residuals(const SpmvDev<double> &A, const double *x, double *y, const double *b,
+                      long long ld, unsigned mask, double *partials, Scalars *slots,
+                      cudaStream_t st);
 // persistent grid of pipeline shape `shape` (< 0 on a CUDA error), and the
 // number of compiled shapes per precision (spmv_cfg.cuh)
 template <typename T>

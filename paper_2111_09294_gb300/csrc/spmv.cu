@@ -34,8 +34,16 @@ namespace xdcg {
 template <typename T, bool RES, int SHAPE>
 __global__ void __launch_bounds__(kSpmvThreads, SpmvCfg<T, SHAPE>::MINB)
 k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__restrict__ b,
-       double *partials, Scalars *sc, int fin, int slot) {
+       double *partials, Scalars *sc, int fin, int slot, SpmvCols cols) {
     using Cfg = SpmvCfg<T, SHAPE>;
+    if (cols.list) {   // several columns in one launch: blockIdx.y picks this block's
+        const int j = (int)(cols.list >> (4 * blockIdx.y) & 15ull) - 1;
+        x += j * cols.ld;
+        y += j * cols.ld;
+        b += j * cols.ld;
+        sc += j;
+        partials += (size_t)j * gridDim.x;
+    }
     constexpr int C = Cfg::C, NS = Cfg::NS, SB = stage_bytes<T, SHAPE>();
     extern __shared__ __align__(128) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -567,9 +575,14 @@ int persistent_grid_of(int nSlicesTotal) {
 
 template <typename T, bool RES, int SHAPE>
 void launch_shape(const SpmvDev<T> &A, const T *x, T *y, const T *b, double *partials,
-                  Scalars *sc, int fin, int slot, cudaStream_t st) {
-    launch_pdl(spmv_kernel<T, RES, SHAPE>(), A.grid, kSpmvThreads, spmv_smem_bytes<T, SHAPE>(), st,
-               A, x, y, b, partials, sc, fin, slot);
+                  Scalars *sc, int fin, int slot, SpmvCols cols, int nCols, cudaStream_t st) {
+    const dim3 grid(A.grid, nCols);
+    if constexpr (SpmvCfg<T, SHAPE>::LEAN)
+        launch_pdl(k_spmv_lean<RES, SHAPE>, grid, kSpmvThreads, spmv_smem_bytes<T, SHAPE>(), st, A,
+                   x, y, b, partials, sc, fin, slot);
+    else
+        launch_pdl(k_spmv<T, RES, SHAPE>, grid, kSpmvThreads, spmv_smem_bytes<T, SHAPE>(), st, A, x,
+                   y, b, partials, sc, fin, slot, cols);
 }
 
 template <typename T>
@@ -604,36 +617,52 @@ int spmv_persistent_grid<double>(int nSlicesTotal, int shape) {
 
 template <typename T, bool RES>
 void launch_spmv_res(const SpmvDev<T> &A, const T *x, T *y, const T *b, double *partials,
-                     Scalars *sc, int fin, int slot, cudaStream_t st) {
+                     Scalars *sc, int fin, int slot, SpmvCols cols, int nCols,
+                     cudaStream_t st) {
     switch (A.shape) {
-        case 1: launch_shape<T, RES, 1>(A, x, y, b, partials, sc, fin, slot, st); return;
-        case 2: launch_shape<T, RES, 2>(A, x, y, b, partials, sc, fin, slot, st); return;
-        case 3: launch_shape<T, RES, 3>(A, x, y, b, partials, sc, fin, slot, st); return;
+        case 1: launch_shape<T, RES, 1>(A, x, y, b, partials, sc, fin, slot, cols, nCols, st); return;
+        case 2: launch_shape<T, RES, 2>(A, x, y, b, partials, sc, fin, slot, cols, nCols, st); return;
+        case 3: launch_shape<T, RES, 3>(A, x, y, b, partials, sc, fin, slot, cols, nCols, st); return;
         case 4:
         case 5:
         case 6:
         case 7:
             if constexpr (SpmvShapes<T>::count > 7) {
                 switch (A.shape) {
-                    case 4: launch_shape<T, RES, 4>(A, x, y, b, partials, sc, fin, slot, st); return;
-                    case 5: launch_shape<T, RES, 5>(A, x, y, b, partials, sc, fin, slot, st); return;
-                    case 6: launch_shape<T, RES, 6>(A, x, y, b, partials, sc, fin, slot, st); return;
-                    default: launch_shape<T, RES, 7>(A, x, y, b, partials, sc, fin, slot, st); return;
+                    case 4: launch_shape<T, RES, 4>(A, x, y, b, partials, sc, fin, slot, cols, nCols, st); return;
+                    case 5: launch_shape<T, RES, 5>(A, x, y, b, partials, sc, fin, slot, cols, nCols, st); return;
+                    case 6: launch_shape<T, RES, 6>(A, x, y, b, partials, sc, fin, slot, cols, nCols, st); return;
+                    default: launch_shape<T, RES, 7>(A, x, y, b, partials, sc, fin, slot, cols, nCols, st); return;
                 }
             }
             break;
         default: break;
     }
-    launch_shape<T, RES, 0>(A, x, y, b, partials, sc, fin, slot, st);
+    launch_shape<T, RES, 0>(A, x, y, b, partials, sc, fin, slot, cols, nCols, st);
 }
 
 template <typename T>
 void launch_spmv(const SpmvDev<T> &A, const T *x, T *y, const T *b, int residual_mode,
                  double *partials, Scalars *sc, int fin, int slot, cudaStream_t st) {
     if (residual_mode)
-        launch_spmv_res<T, true>(A, x, y, b, partials, sc, fin, slot, st);
+        launch_spmv_res<T, true>(A, x, y, b, partials, sc, fin, slot, SpmvCols{0, 0}, 1, st);
     else
-        launch_spmv_res<T, false>(A, x, y, b, partials, sc, fin, slot, st);
+        launch_spmv_res<T, false>(A, x, y, b, partials, sc, fin, slot, SpmvCols{0, 0}, 1, st);
+}
+
+// The residuals b_j - K x_j of the columns in mask (column j at offset j ld) and
+// their squared norms (scratch[0] of slots[j]) in one launch: the blocks of one
+// column after those of another, without a launch's ramp and tail in between (32^3:
+// 267 us for eight columns, 8 x 44 one by one).
+void launch_residuals(const SpmvDev<double> &A, const double *x, double *y, const double *b,
+                      long long ld, unsigned mask, double *partials, Scalars *slots,
+                      cudaStream_t st) {
+    SpmvCols cols{0, ld};
+    int n = 0;
+    for (int j = 0; j < kMaxBatch; ++j)
+        if (mask >> j & 1u) cols.list |= (unsigned long long)(j + 1) << (4 * n++);
+    if (n > 0)
+        launch_spmv_res<double, true>(A, x, y, b, partials, slots, kFinStore, 0, cols, n, st);
 }
 
 template void launch_spmv<double>(const SpmvDev<double> &, const double *, double *,

@@ -64,7 +64,30 @@ __device__ __forceinline__ int sys_of(const int *__restrict__ off, int nSys, int
 // The iteration counts (its, its_j) advance when a column still runs;
 // otherwise the system stops until the host's next replacement.
 // fin 1 (start): rr_j.
-__device__ __forceinline__ void batch_finalize(BatchScalars *bs, int m, int fin, double tot) {
+// in: the column's state, loaded while the sums are formed.
+struct ColumnLoads {
+    double rho = 0.0, rr = 0.0, trig = 0.0, rrRep = 0.0;
+    int its = 0, fault = 0, maxIt = 0;
+    bool runs = false, active = false, repl = false, broken = false;
+    __device__ __forceinline__ void load(const BatchScalars *bs, int m) {
+        const int j = threadIdx.x;
+        if (j >= 32) return;
+        fault = __ldcg(&bs->fault);
+        maxIt = bs->max_it;
+        if (j >= m) return;
+        rho = bs->rho[j];
+        rr = bs->rr[j];
+        trig = bs->trig[j];
+        rrRep = bs->rrRep[j];
+        its = bs->itsc[j];
+        active = bs->active[j] != 0;
+        runs = active && !bs->pend[j];
+        repl = bs->repl[j] != 0;
+        broken = bs->broken[j] != 0;
+    }
+};
+__device__ __forceinline__ void batch_finalize(BatchScalars *bs, int m, int fin, double tot,
+                                               const ColumnLoads &in) {
     const int j = threadIdx.x & 31;
     if (fin != 0) {
         if (j < m) bs->rr[j] = tot;
@@ -73,16 +96,16 @@ __device__ __forceinline__ void batch_finalize(BatchScalars *bs, int m, int fin,
     bool any = false;
     if (j < m) {
         bs->pq[j] = tot;
-        if (!col_runs(bs, j, m)) {
+        if (!in.runs) {
             bs->alpha[j] = 0.0;
         } else {
-            bs->itsc[j] += 1;
+            bs->itsc[j] = in.its + 1;
             if (!(tot > 0.0) || !isfinite(tot)) {
                 bs->alpha[j] = 0.0;
                 bs->broken[j] = 1;
                 bs->pend[j] = 1;
             } else {
-                bs->alpha[j] = bs->rho[j] / tot;
+                bs->alpha[j] = in.rho / tot;
                 any = true;
             }
         }
@@ -366,10 +389,12 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
         blkSum = (double)sum_of_8(w);
     }
     double tot;
-    if (grid_sum_lanes<MB>(blkSum, args.partials, &bs->ticket[0], tot, blk, nblk) &&
+    ColumnLoads in;
+    if (grid_sum_lanes<MB>(blkSum, args.partials, &bs->ticket[0], tot, blk, nblk,
+                           [&] { in.load(bs, m); }) &&
         threadIdx.x < 32) {
-        if (!bs->fault)
-            batch_finalize(bs, m, fin, tot);
+        if (!in.fault)
+            batch_finalize(bs, m, fin, tot, in);
         else if (threadIdx.x == 0)
             bs->done = kFault;
     }
@@ -622,9 +647,22 @@ __device__ __forceinline__ bool restrict_b_unit(const RestrictBArgs &a, int unit
             if ((int)threadIdx.x < MB * M) {
                 const int jj = threadIdx.x / M, c = threadIdx.x % M;
                 double zsum = 0.0, wsum = 0.0;
-                for (int v = u0; v < u0 + nu; ++v) {
-                    zsum += __ldcg(unitPart + ((size_t)v * MB + jj) * 24 + c);
-                    wsum += __ldcg(unitPart + ((size_t)v * MB + jj) * 24 + M + c);
+                const double *up = unitPart + ((size_t)u0 * MB + jj) * 24 + c;
+                for (int v = 0; v < nu; v += 4) {   // four units' loads in flight
+                    double zv[4], wv[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        zv[i] = v + i < nu ? __ldcg(up + (size_t)(v + i) * MB * 24) : 0.0;
+                        wv[i] = v + i < nu ? __ldcg(up + (size_t)(v + i) * MB * 24 + M) : 0.0;
+                    }
+                    zsum = v == 0 ? zv[0] : zsum + zv[0];
+                    wsum = v == 0 ? wv[0] : wsum + wv[0];
+#pragma unroll
+                    for (int i = 1; i < 4; ++i)
+                        if (v + i < nu) {
+                            zsum += zv[i];
+                            wsum += wv[i];
+                        }
                 }
                 G[(size_t)(c0 + c) * MB + jj] = zsum - wsum;
                 G32[(size_t)jj * a.gld + c0 + c] = (float)(zsum - wsum);
@@ -654,17 +692,20 @@ __device__ __forceinline__ void restrict_b_body(const RestrictBArgs &a, int blk,
     // lane j of warp 0 adds column j's ||r||^2
     const double rr = threadIdx.x < MB ? (double)rrs[threadIdx.x] : 0.0;
     double tot;
-    if (grid_sum_lanes<MB>(rr, a.partials, &bs->ticket[2], tot, blk, nblk) && threadIdx.x < 32) {
+    ColumnLoads in;
+    if (grid_sum_lanes<MB>(rr, a.partials, &bs->ticket[2], tot, blk, nblk,
+                           [&] { in.load(bs, m); }) &&
+        threadIdx.x < 32) {
         const int j = threadIdx.x;   // one column per lane
         if (mode == 1) {
-            if (j < m && bs->repl[j]) bs->rr[j] = tot;
+            if (in.repl) bs->rr[j] = tot;
             return;
         }
         bool any = false;
-        if (j < m && col_runs(bs, j, m)) {
+        if (in.runs) {
             bs->rr[j] = tot;
-            bool hold = tot <= bs->trig[j] || !isfinite(tot);
-            if (bs->itsc[j] >= bs->max_it) {
+            bool hold = tot <= in.trig || !isfinite(tot);
+            if (in.its >= in.maxIt) {
                 hold = true;
                 bs->last[j] = 1;
             }
@@ -832,18 +873,21 @@ __device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int
         for (int o = MB; o < 32; o <<= 1) pj += __shfl_xor_sync(0xffffffffu, pj, o);
     }
     double tot;
-    if (grid_sum_lanes<MB>(pj, a.partials, &bs->ticket[3], tot, blk, nblk) && threadIdx.x < 32) {
+    ColumnLoads in;
+    if (grid_sum_lanes<MB>(pj, a.partials, &bs->ticket[3], tot, blk, nblk,
+                           [&] { in.load(bs, m); }) &&
+        threadIdx.x < 32) {
         const int j = threadIdx.x;   // one column per lane
-        if (bs->fault) {
+        if (in.fault) {
             if (j == 0) bs->done = kFault;
         } else if (mode != 0 && j < m &&
-                   (mode == 2 ? col_runs(bs, j, m) : (mode == 1 || bs->repl[j]))) {
-            const double rho_new = bs->rr[j] + tot;
-            if (mode == 1 || !bs->active[j] ||
-                (mode == 3 && (bs->broken[j] || bs->rr[j] > 4.0 * bs->rrRep[j])))
+                   (mode == 2 ? in.runs : (mode == 1 || in.repl))) {
+            const double rho_new = in.rr + tot;
+            if (mode == 1 || !in.active ||
+                (mode == 3 && (in.broken || in.rr > 4.0 * in.rrRep)))
                 bs->beta[j] = 0.0;
             else
-                bs->beta[j] = rho_new / bs->rho[j];
+                bs->beta[j] = rho_new / in.rho;
             bs->rho[j] = rho_new;
             if (mode == 3) bs->broken[j] = 0;
         }

@@ -190,7 +190,7 @@ k_block_apply(BlkDev<T> B, const T *__restrict__ r, T *__restrict__ y, double *p
         }
     }
     double tot;
-    if (grid_sum<T>(part, partials, &sc->ticket[1], tot) && threadIdx.x == 0) sc->ry = tot;
+    if (grid_sum<T>(part, partials, &sc->ticket[1], tot, [] {}) && threadIdx.x == 0) sc->ry = tot;
 }
 
 template <typename T>
@@ -224,7 +224,9 @@ k_update_plain(T *u, T *r, const T *p, const T *q, long long n, int mode, double
         v[0] = fma(ri, ri, v[0]);
     }
     double tot;
-    if (grid_sum<T>(v[0], partials, &sc->ticket[2], tot) && threadIdx.x == 0) {
+    FinLoads in;
+    if (grid_sum<T>(v[0], partials, &sc->ticket[2], tot, [&] { in.load(sc); }) &&
+        threadIdx.x == 0) {
         sc->rr = tot;
         if (sc->hist && sc->its < sc->histCap) sc->hist[sc->its] = tot;
         if (tot <= sc->tol2ff)

@@ -191,7 +191,7 @@ __device__ __forceinline__ void coarse_scalars(double blk, int rowBlk, int mode,
                                                double *partials, const ResidualSums &sums,
                                                Scalars *sc) {
     if (rowBlk < 0) {
-        if (sums.values == 2) {
+        if (THREADS == kThreads && sums.values == 2) {
             const double t = sum_partials<2>(sums.part, &sc->ticket[2], sums.n);
             if (threadIdx.x == 0) sc->rr = t;
             if (threadIdx.x == 1) sc->ry = t;

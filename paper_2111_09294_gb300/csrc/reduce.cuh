@@ -87,29 +87,90 @@ __device__ __forceinline__ float sum_of_8(const float (&x)[8]) {
 
 // The last block's share of a grid-wide sum: value i of the nblk blocks'
 // partials (partials[i * nblk + b]) added by one warp, its lanes striding
-// over the blocks with four accumulators each, then across the lanes (a fixed
-// order, and FP64 work spread over the warps: FP64 arithmetic is slow here).
-// Thread i < NV gets total i; thread 0 resets the ticket.
+// over the blocks with four accumulators each (lane l: rounds of 128 partials
+// while l + 96 is in range, the rest into the first accumulator), then across the
+// lanes (a fixed order, and FP64 work spread over the warps: FP64 arithmetic is
+// slow here).  Thread i < NV gets total i; thread 0 resets the ticket.
+//
+// This is the tail of its kernel, on one SM while the others wait: four rounds
+// of loads are in flight at once (one round trip to L2 instead of one per round),
+// the first partial of an accumulator is not added to a zero, and where the
+// block has four warps per value each takes one accumulator.  Solves at 1e-8, this
+// and what the last block reads next loaded beside the sum: 8 columns at 8^3 3.40 ->
+// 3.22 ms, at 32^3 8.63 -> 8.52; one mixed one at 8^3 1.47 -> 1.42, at 32^3 3.66 ->
+// 3.55; FP64 at 32^3 9.46 -> 9.32.
 template <int NV>
 __device__ __forceinline__ double sum_partials(const double *partials, unsigned int *ticket,
                                                int nblk) {
     __shared__ double fin[NV];
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int i = w; i < NV; i += nw) {
-        const double *p = partials + (size_t)i * nblk;
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        int b = l;
-        for (; b + 96 < nblk; b += 128) {
-            s0 += __ldcg(p + b);
-            s1 += __ldcg(p + b + 32);
-            s2 += __ldcg(p + b + 64);
-            s3 += __ldcg(p + b + 96);
-        }
-        for (; b < nblk; b += 32) s0 += __ldcg(p + b);
-        double s = (s0 + s1) + (s2 + s3);
+    const int rounds = nblk > l + 96 ? (nblk - l - 96 + 127) >> 7 : 0;
+    if (NV <= 2 && nw >= 4 * NV) {
+        __shared__ double acc[NV <= 2 ? 4 * NV : 1][32];
+        if (w < 4 * NV) {
+            const int q = w & 3;
+            const double *p = partials + (size_t)(w >> 2) * nblk + l;
+            double x[3], s = 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (l == 0) fin[i] = s;
+            for (int t = 0; t < 3; ++t) {
+                const int b = 128 * rounds + 32 * t;
+                x[t] = q == 0 && l + b < nblk ? __ldcg(p + b) : 0.0;
+            }
+            for (int r0 = 0; r0 < rounds; r0 += 4) {
+                double v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    v[u] = r0 + u < rounds ? __ldcg(p + 128 * (r0 + u) + 32 * q) : 0.0;
+                s = r0 == 0 ? v[0] : s + v[0];
+#pragma unroll
+                for (int u = 1; u < 4; ++u)
+                    if (r0 + u < rounds) s += v[u];
+            }
+#pragma unroll
+            for (int t = 0; t < 3; ++t)
+                if (q == 0 && l + 128 * rounds + 32 * t < nblk) s += x[t];
+            acc[w % (NV <= 2 ? 4 * NV : 1)][l] = s;
+        }
+        __syncthreads();
+        if (w < NV) {
+            const int i = NV <= 2 ? 4 * w : 0;
+            double s = (acc[i][l] + acc[i + 1][l]) + (acc[i + 2][l] + acc[i + 3][l]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (l == 0) fin[w] = s;
+        }
+    } else {
+        for (int i = w; i < NV; i += nw) {
+            const double *p = partials + (size_t)i * nblk + l;
+            double x[3], s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                const int b = 128 * rounds + 32 * t;
+                x[t] = l + b < nblk ? __ldcg(p + b) : 0.0;
+            }
+            for (int r0 = 0; r0 < rounds; r0 += 4) {
+                double v[4][4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        v[u][q] = r0 + u < rounds ? __ldcg(p + 128 * (r0 + u) + 32 * q) : 0.0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s[q] = r0 == 0 ? v[0][q] : s[q] + v[0][q];
+#pragma unroll
+                for (int u = 1; u < 4; ++u)
+                    if (r0 + u < rounds)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) s[q] += v[u][q];
+            }
+#pragma unroll
+            for (int t = 0; t < 3; ++t)
+                if (l + 128 * rounds + 32 * t < nblk) s[0] += x[t];
+            double t = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (l == 0) fin[i] = t;
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) *ticket = 0u;
@@ -121,10 +182,12 @@ __device__ __forceinline__ double sum_partials(const double *partials, unsigned 
 // reduction, over the blocks blk = 0 .. nblk - 1 of one reduction (the launch's, or
 // one system's share of a launch over several systems); in the last block to
 // finish, which returns true, the totals come back to the same lanes.  Every
-// thread of the block calls it.  partials: NV * nblk doubles.
-template <int NV>
+// thread of the block calls it.  partials: NV * nblk doubles.  loads(): run by the
+// last block before the sum, for what it reads next (the latency then passes
+// beside the sum).
+template <int NV, typename F>
 __device__ __forceinline__ bool grid_sum_lanes(double v, double *partials, unsigned int *ticket,
-                                               double &tot, int blk, int nblk) {
+                                               double &tot, int blk, int nblk, F loads) {
     __shared__ bool last;
     if (threadIdx.x < 32) {
         if ((int)threadIdx.x < NV) partials[(size_t)threadIdx.x * nblk + blk] = v;
@@ -135,6 +198,7 @@ __device__ __forceinline__ bool grid_sum_lanes(double v, double *partials, unsig
     __syncthreads();
     if (!last) return false;
     __threadfence();
+    loads();
     tot = sum_partials<NV>(partials, ticket, nblk);
     return true;
 }
@@ -194,10 +258,10 @@ __device__ __forceinline__ double block_total_t0(const float2 *partials, int n) 
 
 // Grid-wide sum of one value per thread over the launch's blocks.  Returns true
 // in exactly one of them (the last to finish), where thread 0 then holds the
-// FP64 total in tot.  partials: one double per block.
-template <typename A>
+// FP64 total in tot.  partials: one double per block; loads() as in grid_sum_lanes.
+template <typename A, typename F>
 __device__ __forceinline__ bool grid_sum(A v, double *partials, unsigned int *ticket,
-                                         double &tot) {
+                                         double &tot, F loads) {
     __shared__ bool last;
     A s[1] = {v};
     block_sum<A, 1>(s);
@@ -209,6 +273,7 @@ __device__ __forceinline__ bool grid_sum(A v, double *partials, unsigned int *ti
     __syncthreads();
     if (!last) return false;
     __threadfence();
+    loads();
     tot = sum_partials<1>(partials, ticket, (int)gridDim.x);
     return true;
 }
@@ -217,20 +282,33 @@ __device__ __forceinline__ bool grid_sum(A v, double *partials, unsigned int *ti
 // The order of the sum is that of 256 threads whatever THREADS: slot t = 0 ..
 // 255 adds partials t, t + 256, ..., then the tree over the 32 slots of a warp and
 // the tree over the eight warps; a thread of a smaller block takes 256 / THREADS
-// slots.
+// slots, with two rounds of loads in flight after the first.
 template <int THREADS>
 __device__ __forceinline__ double sum_slots(const double *p, int n) {
-    constexpr int Q = kThreads / THREADS;
+    constexpr int Q = kThreads / THREADS, U = 2;
     static_assert(Q == 1 || Q == 4, "");
     __shared__ double sums[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double s[Q];
 #pragma unroll
-    for (int q = 0; q < Q; ++q) s[q] = 0.0;
-    for (int b = threadIdx.x; b < n; b += kThreads)
+    for (int q = 0; q < Q; ++q)
+        s[q] = (int)threadIdx.x + q * THREADS < n ? __ldcg(p + threadIdx.x + q * THREADS) : 0.0;
+#pragma unroll 1
+    for (int b = threadIdx.x + kThreads; b < n; b += U * kThreads) {
+        double v[U][Q];
 #pragma unroll
-        for (int q = 0; q < Q; ++q)
-            if (b + q * THREADS < n) s[q] += __ldcg(p + b + q * THREADS);
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int i = b + u * kThreads + q * THREADS;
+                v[u][q] = i < n ? __ldcg(p + i) : 0.0;
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (b + u * kThreads + q * THREADS < n) s[q] += v[u][q];
+    }
     int o = 16;
     if (Q == 4) {   // halving exchanges: lanes 8 q .. 8 q + 7 keep the sums of slot set q
 #pragma unroll
@@ -286,20 +364,33 @@ __device__ __forceinline__ void report(const Scalars *sc) {
     p->rr[sc->its % kRing] = v;
 }
 
-// Shared last-block actions on the scalar block.
-__device__ __forceinline__ void finalize(Scalars *sc, int fin, int slot, double val) {
+// Shared last-block actions on the scalar block.  FinLoads: what they read,
+// loaded while the sum is formed (grid_sum's loads()).
+struct FinLoads {
+    double rho = 0.0, tol2ff = 0.0;
+    int its = 0, fault = 0;
+    __device__ __forceinline__ void load(const Scalars *sc) {
+        if (threadIdx.x != 0) return;
+        rho = sc->rho;
+        tol2ff = sc->tol2ff;
+        its = sc->its;
+        fault = __ldcg(&sc->fault);
+    }
+};
+__device__ __forceinline__ void finalize(Scalars *sc, int fin, int slot, double val,
+                                         const FinLoads &in) {
     if (fin == kFinAlpha) {
         sc->pq = val;
-        sc->its += 1;
+        sc->its = in.its + 1;
         if (!(val > 0.0) || !isfinite(val)) {
             sc->done = kBreakdown;
         } else {
-            sc->alpha = sc->rho / val;
+            sc->alpha = in.rho / val;
         }
     } else if (fin == kFinRR) {
         sc->rr = val;
         if (sc->hist && sc->histCap > 0) sc->hist[0] = val;
-        if (val <= sc->tol2ff) sc->done = kConverged;
+        if (val <= in.tol2ff) sc->done = kConverged;
     } else {
         sc->scratch[slot] = val;
     }

@@ -271,11 +271,13 @@ k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__rest
         return;
     }
     double tot;
-    if (grid_sum<T>(part[0], partials, &sc->ticket[0], tot) && threadIdx.x == 0) {
-        if (sc->fault)
+    FinLoads in;
+    if (grid_sum<T>(part[0], partials, &sc->ticket[0], tot, [&] { in.load(sc); }) &&
+        threadIdx.x == 0) {
+        if (in.fault)
             sc->done = kFault;
         else
-            finalize(sc, fin, slot, tot);
+            finalize(sc, fin, slot, tot, in);
     }
 }
 
@@ -535,11 +537,13 @@ k_spmv_lean(SpmvDev<float> A, const float *__restrict__ x, float *__restrict__ y
         return;
     }
     double tot;
-    if (grid_sum<float>(part[0], partials, &sc->ticket[0], tot) && threadIdx.x == 0) {
-        if (sc->fault)
+    FinLoads in;
+    if (grid_sum<float>(part[0], partials, &sc->ticket[0], tot, [&] { in.load(sc); }) &&
+        threadIdx.x == 0) {
+        if (in.fault)
             sc->done = kFault;
         else
-            finalize(sc, fin, slot, tot);
+            finalize(sc, fin, slot, tot, in);
     }
 }
 
@@ -694,8 +698,10 @@ k_dot(const T *__restrict__ a, const T *__restrict__ b, long long n, double *par
          i += (long long)gridDim.x * blockDim.x)
         part[0] = fma(a[i], b[i], part[0]);
     double tot;
-    if (grid_sum<T>(part[0], partials, &sc->ticket[1], tot) && threadIdx.x == 0)
-        finalize(sc, fin, slot, tot);
+    FinLoads in;
+    if (grid_sum<T>(part[0], partials, &sc->ticket[1], tot, [&] { in.load(sc); }) &&
+        threadIdx.x == 0)
+        finalize(sc, fin, slot, tot, in);
 }
 
 template <typename T>

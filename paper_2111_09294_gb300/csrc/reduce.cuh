@@ -278,6 +278,60 @@ __device__ __forceinline__ bool grid_sum(A v, double *partials, unsigned int *ti
     return true;
 }
 
+// grid_sum with the bits it has for 256 threads per block, from a launch of twice
+// as many blocks of 128: groups of eight warps (two blocks), each warp's sum in
+// partials (8 doubles per group), which the last block first adds within the
+// groups by block_sum's tree.  Thread t of it takes groups t, t + 128, ...: in
+// sum_partials' order warp q's are accumulator q's, and the last, incomplete
+// round belongs to the first accumulator.
+template <typename F>
+__device__ __forceinline__ bool grid_sum_halves(double v, double *partials, unsigned int *ticket,
+                                                double &tot, F loads) {
+    __shared__ bool last;
+    __shared__ double acc[4][32], rest[4][32];
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, n = (int)gridDim.x / 2;
+    double s[1] = {v};
+    warp_sum<double, 1>(s);
+    if (l == 0) partials[blockIdx.x * 4 + w] = s[0];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    loads();
+    const int rounds = n > l + 96 ? (n - l - 96 + 127) >> 7 : 0;
+    double a = 0.0, r = 0.0;
+#pragma unroll 1
+    for (int i = 0; i <= rounds; ++i) {
+        const int g = threadIdx.x + 128 * i;
+        if (g >= n) break;
+        const double2 *y = reinterpret_cast<const double2 *>(partials) + 4 * g;
+        const double2 y0 = __ldcg(y), y2 = __ldcg(y + 1), y4 = __ldcg(y + 2), y6 = __ldcg(y + 3);
+        const double t = ((y0.x + y4.x) + (y2.x + y6.x)) + ((y0.y + y4.y) + (y2.y + y6.y));
+        if (i == rounds)
+            r = t;
+        else
+            a = i == 0 ? t : a + t;
+    }
+    acc[w][l] = a;
+    rest[w][l] = r;
+    __syncthreads();
+    if (w == 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (l + 128 * rounds + 32 * q < n) a += rest[q][l];
+        a = (a + acc[1][l]) + (acc[2][l] + acc[3][l]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (l == 0) *ticket = 0u;
+    }
+    tot = a;
+    return true;
+}
+
 // Sum of n block partials by one block of THREADS threads, valid in thread 0.
 // The order of the sum is that of 256 threads whatever THREADS: slot t = 0 ..
 // 255 adds partials t, t + 256, ..., then the tree over the 32 slots of a warp and

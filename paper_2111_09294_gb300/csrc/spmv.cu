@@ -31,8 +31,18 @@ namespace xdcg {
 // next: the first 32 slices' extents are read into shared memory at kernel
 // start (one slice per lane), and a slice's row indices are loaded when the
 // slice begins, its x (or b) entries one stage later, for use when it ends.
-template <typename T, bool RES, int SHAPE>
-__global__ void __launch_bounds__(kSpmvThreads, SpmvCfg<T, SHAPE>::MINB)
+//
+// W warps per launched block.  The slice ranges and the dot belong to groups of
+// kSpmvWarps warps; W = kSpmvWarps launches a group as a block.  FP64 arithmetic
+// bounds the FP64 product (64 cycles per warp instruction on an SM partition,
+// nine instructions per step), so a matrix that does not fill the SMs with whole
+// groups is launched in half groups: four warps take the four partitions of an SM,
+// where eight share them, and the leftover blocks are half as long.  Their last
+// block then adds the warps' sums, in the group's order.  FP64 solves at
+// 1e-8: 24^3 (319 groups) 5.46 ms in whole groups, 5.26 in halves; 8^3 2.946 and 2.933;
+// 32^3 (416 groups) 9.34 both.
+template <typename T, bool RES, int SHAPE, int W>
+__global__ void __launch_bounds__(32 * W, SpmvCfg<T, SHAPE>::MINB * (kSpmvWarps / W))
 k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__restrict__ b,
        double *partials, Scalars *sc, int fin, int slot, SpmvCols cols) {
     using Cfg = SpmvCfg<T, SHAPE>;
@@ -48,14 +58,14 @@ k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__rest
     extern __shared__ __align__(128) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char *ring = smem + (size_t)warp * NS * SB;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kSpmvWarps * NS * SB) + warp * NS;
-    int *meta = reinterpret_cast<int *>(smem + (size_t)kSpmvWarps * NS * (SB + 8)) + warp * NS * 3;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)W * NS * SB) + warp * NS;
+    int *meta = reinterpret_cast<int *>(smem + (size_t)W * NS * (SB + 8)) + warp * NS * 3;
     const int nS = A.S.nSlices;
-    const int gw = blockIdx.x * kSpmvWarps + warp;
+    const int gw = blockIdx.x * W + warp;
     const int sFirst = A.warpSlice[gw], sEnd = A.warpSlice[gw + 1];
     // extents of the warp's first 32 slices (set-up data)
-    __shared__ long long tBase[kSpmvWarps][32];
-    __shared__ int tSteps[kSpmvWarps][32];
+    __shared__ long long tBase[W][32];
+    __shared__ int tSteps[W][32];
     if (sFirst + lane < sEnd) {
         const int g = sFirst + lane;
         const SellDev<T> &P = g < nS ? A.S : A.X;
@@ -262,18 +272,23 @@ k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__rest
         for (; k < issued; ++k) mbar_wait(bars + k % NS, (uint32_t)(k / NS) & 1u, drain);
         __syncwarp();
     }
-    if (fin == kFinDefer) {
-        // the next kernel adds the blocks' sums (block_total_t0); a failed
-        // wait is in sc->fault, which it reads too
-        block_sum<T, 1>(part);
-        if (threadIdx.x == 0)
-            reinterpret_cast<float2 *>(partials)[blockIdx.x] = df_of((double)part[0]);
-        return;
-    }
-    double tot;
     FinLoads in;
-    if (grid_sum<T>(part[0], partials, &sc->ticket[0], tot, [&] { in.load(sc); }) &&
-        threadIdx.x == 0) {
+    double tot;
+    bool last;
+    if constexpr (W == kSpmvWarps) {
+        if (fin == kFinDefer) {
+            // the next kernel adds the blocks' sums (block_total_t0); a failed
+            // wait is in sc->fault, which it reads too
+            block_sum<T, 1>(part);
+            if (threadIdx.x == 0)
+                reinterpret_cast<float2 *>(partials)[blockIdx.x] = df_of((double)part[0]);
+            return;
+        }
+        last = grid_sum<T>(part[0], partials, &sc->ticket[0], tot, [&] { in.load(sc); });
+    } else {
+        last = grid_sum_halves(part[0], partials, &sc->ticket[0], tot, [&] { in.load(sc); });
+    }
+    if (last && threadIdx.x == 0) {
         if (in.fault)
             sc->done = kFault;
         else
@@ -553,7 +568,7 @@ constexpr auto spmv_kernel() {
     if constexpr (SpmvCfg<T, SHAPE>::LEAN)
         return k_spmv_lean<RES, SHAPE>;
     else
-        return k_spmv<T, RES, SHAPE>;
+        return k_spmv<T, RES, SHAPE, kSpmvWarps>;
 }
 
 // Persistent grid of a shape: its resident blocks per SM times the SMs (at
@@ -584,9 +599,22 @@ void launch_shape(const SpmvDev<T> &A, const T *x, T *y, const T *b, double *par
     if constexpr (SpmvCfg<T, SHAPE>::LEAN)
         launch_pdl(k_spmv_lean<RES, SHAPE>, grid, kSpmvThreads, spmv_smem_bytes<T, SHAPE>(), st, A,
                    x, y, b, partials, sc, fin, slot);
-    else
-        launch_pdl(k_spmv<T, RES, SHAPE>, grid, kSpmvThreads, spmv_smem_bytes<T, SHAPE>(), st, A, x,
-                   y, b, partials, sc, fin, slot, cols);
+    else if constexpr (std::is_same<T, double>::value) {
+        // half groups where whole ones leave part of the SMs' block slots empty (and
+        // the smallest array of partial sums a caller has takes one per warp)
+        if (!cols.list && A.grid < SpmvCfg<T, SHAPE>::MINB * device_sm_count() &&
+            A.grid * kSpmvWarps <= XDCG_NOALLOC_MAX_BLOCKS) {
+            launch_pdl(k_spmv<T, RES, SHAPE, kSpmvWarps / 2>, dim3(2 * A.grid), kSpmvThreads / 2,
+                       spmv_smem_bytes<T, SHAPE>() / 2, st, A, x, y, b, partials, sc, fin, slot,
+                       cols);
+            return;
+        }
+        launch_pdl(spmv_kernel<T, RES, SHAPE>(), grid, kSpmvThreads, spmv_smem_bytes<T, SHAPE>(),
+                   st, A, x, y, b, partials, sc, fin, slot, cols);
+    } else {
+        launch_pdl(spmv_kernel<T, RES, SHAPE>(), grid, kSpmvThreads, spmv_smem_bytes<T, SHAPE>(),
+                   st, A, x, y, b, partials, sc, fin, slot, cols);
+    }
 }
 
 template <typename T>

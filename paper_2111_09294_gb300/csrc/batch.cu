@@ -333,7 +333,7 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
                     } else if (t + 1 < C && t + 1 < curN) {
                         gather(cslot, t + 1, 0, xn);
                     } else if (haveN) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(bars + nslot, npar, deadline));
+                        ok = __all_sync(0xffffffffu, mbar_wait_next(bars + nslot, npar, deadline));
                         if (ok) gather(nslot, 0, 0, xn);
                     }
                     const float *v = vs + t * 288 + q * SPP + sl0;

@@ -210,7 +210,7 @@ k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__rest
         int nb = 0;
         if (k + 1 < issued) {
             const int s1 = (k + 1) % NS;
-            ok = __all_sync(0xffffffffu, mbar_wait(bars + s1, (uint32_t)((k + 1) / NS) & 1u, deadline));
+            ok = __all_sync(0xffffffffu, mbar_wait_next(bars + s1, (uint32_t)((k + 1) / NS) & 1u, deadline));
             if (!ok) break;
             nb = meta[s1 * 3 + 2];
             gather(s1, nb, xb);
@@ -498,7 +498,7 @@ k_spmv_lean(SpmvDev<float> A, const float *__restrict__ x, float *__restrict__ y
         const int nslot = cslot + 1 == NS ? 0 : cslot + 1;
         const uint32_t npar = nslot == 0 ? cpar ^ 1u : cpar;
         if (haveN) {
-            ok = __all_sync(0xffffffffu, mbar_wait(bars + nslot, npar, deadline));
+            ok = __all_sync(0xffffffffu, mbar_wait_next(bars + nslot, npar, deadline));
             if (!ok) return false;
             gather(nslot, nxtN, xn);
         }

@@ -683,7 +683,7 @@ def run_ours(args):
                 "graph_launches_per_solve_mixed": inf_mg[-1]["n_graph_launches"],
                 "rel_res_true_mixed": max(i["rel_res_true"] for i in inf_mg),
                 "same_bits_as_stream_launches": same,
-                "note": "8 iterations per graph launch; timed like the value"}
+                "note": "4 iterations per graph launch; timed like the value"}
 
     def iteration_gbs():
         # effective bandwidth of whole iterations: one iteration's algorithmic

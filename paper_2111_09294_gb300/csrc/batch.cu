@@ -520,7 +520,7 @@ __device__ __forceinline__ void row_times(const float *z, float rn, float *acc) 
 // The unit's rows of Z~ and W~ and its dof map, shared by the columns, are
 // copied into shared memory before the wait for the product (set-up data);
 // four rows' entries of r, q, p and u are in flight at a time.  8 columns at
-// 32^3 (599 units): 30.4 us before, 18.6 now (four blocks
+// 32^3 (599 units): 30.4 us before, 17.5 now (four blocks
 // per SM).
 template <int MB, int M>
 __device__ __forceinline__ bool restrict_b_unit(const RestrictBArgs &a, int unit, float *stage,
@@ -798,7 +798,7 @@ __device__ __forceinline__ void coarse_load_e(const float *Eb, int k, int rLast,
 // blocks find it after the first.  The partial sums are reduced over the lanes,
 // then over the warps in order.  8 columns, k =
 // 3150: 29.9 us before (G staged by each warp in shared memory through bulk
-// copies and barriers), 24.2 now (three blocks of 80 registers per SM; four of 64
+// copies and barriers), 22.1 now (three blocks of 80 registers per SM; four of 64
 // spill, 39).
 template <int MB, int V>
 __device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int nblk) {

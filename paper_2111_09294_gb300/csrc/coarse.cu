@@ -313,9 +313,9 @@ k_coarse(const double *__restrict__ Einv, int k, const double *__restrict__ g,
 // over the SMs and stay resident together.
 //
 // k = 3240 (42 MB of E^-1, from L2): 17.9 us before (a row per two warps, g read
-// for every row, few loads in flight), 15.9 now; k = 3150 (4-byte loads):
-// 16.0 before, 15.2 now; k = 60: 8.6 before,
-// 10.0 now.
+// for every row, few loads in flight), 14.4 now; k = 3150 (4-byte loads):
+// 16.0 before, 14.5 now; k = 60: 8.6 before, 10.3 now (it now ends the iteration's
+// sums as well, which the restriction did before).
 constexpr int kCoarse32Rows = 4, kCoarse32Threads = 64;
 
 template <int V>

@@ -931,9 +931,11 @@ void launch_coarse_b(const CoarseBArgs &a, cudaStream_t st) {
 // residual buffer.
 //
 // A thread's rows are all in flight at once: their rows of Z~, and in an
-// iteration their entries of y and p, which no kernel still running writes (nor
-// the count that picks y's buffer), before the wait for the coarse solve.  8
-// columns at 32^3: 9.4 us before, 9.2 now.
+// iteration that runs the system their entries of y and p, before the wait for
+// the coarse solve.  No kernel still running writes those, nor the count that
+// picks y's buffer; but in a launch over several systems a held system's
+// replacement, on a stream of its own, writes all three, so the gate's go
+// decides first.  8 columns at 32^3: 9.4 us before, 9.2 now.
 template <int MB, int M>
 __device__ __forceinline__ void prolong_b_unit(const ProlongBArgs &a, int unit) {
     constexpr int kRowStep = kThreads / MB, R = (kProlongRowsBatch + kRowStep - 1) / kRowStep;
@@ -954,7 +956,7 @@ __device__ __forceinline__ void prolong_b_unit(const ProlongBArgs &a, int unit) 
             z[i][c] = r < re ? ld_keep(Z + (size_t)c * RO + r, keep) : 0.0f;
     }
     auto load_vectors = [&]() {
-        const float *y = (bs->its & 1) ? a.rB : a.rA;
+        const float *y = (ld_early(&bs->its) & 1) ? a.rB : a.rA;
 #pragma unroll
         for (int i = 0; i < R; ++i) {
             const int r = rb + i * kRowStep;
@@ -963,7 +965,10 @@ __device__ __forceinline__ void prolong_b_unit(const ProlongBArgs &a, int unit) 
             pv[i] = r < re && (mode == 0 || mode == 3) ? a.p[e] : 0.0f;
         }
     };
-    if (mode == 0) load_vectors();
+    // (done may be stale; the read after the wait decides)
+    const bool early =
+        mode == 0 && ld_early(&bs->go) != 0 && ld_early(&bs->done) == kRunning;
+    if (early) load_vectors();
     pdl_wait();
     if (!batch_runs(bs, mode == 0)) return;
     bool leaves = false;
@@ -973,7 +978,7 @@ __device__ __forceinline__ void prolong_b_unit(const ProlongBArgs &a, int unit) 
         if (j >= a.m || !bs->repl[j]) return;
         leaves = !bs->active[j];
     }
-    if (mode != 0) load_vectors();
+    if (!early) load_vectors();
     const float beta = (mode == 0 || mode == 3) && !leaves ? (float)bs->beta[j] : 0.0f;
     float nv[M];
 #pragma unroll

@@ -36,6 +36,16 @@ __device__ __forceinline__ float4 ld_keep(const float4 *a, uint64_t pol) {
     return v;
 }
 
+// What a kernel reads before its wait for the kernel before it (pdl.cuh) and is
+// not set-up data: from L2, where everything that a finished kernel wrote is.
+// A plain load might find an older line in the SM's L1, since the wait, which
+// makes earlier writes visible, has yet to come.  Not moved across the wait.
+__device__ __forceinline__ int ld_early(const int *a) {
+    int v;
+    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
+    return v;
+}
+
 // asynchronous 4-byte copy into shared memory with the same policy; a thread
 // that reads back only what it copied itself needs no barrier, just the wait
 __device__ __forceinline__ void cp_keep(float *smem, const float *a, uint64_t pol) {

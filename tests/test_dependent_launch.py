@@ -1,0 +1,55 @@
+"""What the kernels may touch before they wait for the kernel before them
+(programmatic dependent launch), checked on the sources: a mistake here is a
+race that a run shows rarely or never, so no run is asked to show it."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2111_09294_gb300", "csrc")
+
+
+def functions():
+    """(file, name, parameters, body) of every function, comments removed."""
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        src = re.sub(r"/\*.*?\*/|//[^\n]*", "", open(path).read(), flags=re.S)
+        for m in re.finditer(r"^(?:__global__|__device__|template|static|inline|void)[^;{}]*?"
+                             r"(\w+)\(((?:[^(){};]|\([^(){};]*\))*)\)\s*(?:const\s*)?\{",
+                             src, flags=re.M):
+            depth, i = 1, m.end()
+            while depth:
+                depth += {"{": 1, "}": -1}.get(src[i], 0)
+                i += 1
+            yield os.path.basename(path), m.group(1), m.group(2), src[m.end():i - 1]
+
+
+def before_wait():
+    """(file, name, text before the first wait) of the functions that wait."""
+    return [(f, n, b[:b.index("pdl_wait()")]) for f, n, _, b in functions() if "pdl_wait()" in b]
+
+
+def test_every_waiting_kernel_is_found():
+    names = {n for _, n, _ in before_wait()}
+    assert {"k_spmv", "k_spmv_lean", "spmm_body", "k_update", "k_restrict", "prolong_box",
+            "restrict_update_unit", "prolong_rows_unit", "k_coarse", "k_coarse32",
+            "restrict_b_unit", "coarse_b_body", "prolong_b_unit", "k_block_apply",
+            "k_renumber"} <= names
+
+
+# the run's scalars change while kernels run: before the wait they are read from
+# L2 only, and only to decide whether to start loading
+@pytest.mark.parametrize("where", before_wait(), ids=lambda w: f"{w[0]}:{w[1]}")
+def test_scalars_before_the_wait_come_from_l2(where):
+    plain = re.sub(r"(?:ld_early|__ldcg)\(&(?:bs|sc)->\w+\)", "", where[2])
+    assert not re.search(r"\b(?:bs|sc)->", plain), where[:2]
+
+
+def test_a_held_system_is_not_read_before_the_wait():
+    # in a launch over several systems the gate's go says whether a replacement
+    # may be writing the system's vectors
+    text, = [t for _, n, t in before_wait() if n == "prolong_b_unit"]
+    early = re.search(r"const bool early\s*=\s*([^;]*);\s*if \(early\) load_vectors\(\);", text)
+    assert early and "ld_early(&bs->go)" in early.group(1)
+    assert text.count("load_vectors()") == 1

@@ -961,8 +961,8 @@ __device__ __forceinline__ void prolong_b_unit(const ProlongBArgs &a, int unit) 
         for (int i = 0; i < R; ++i) {
             const int r = rb + i * kRowStep;
             const size_t e = (size_t)r * MB + j;
-            yv[i] = r < re && mode != 1 ? y[e] : 0.0f;
-            pv[i] = r < re && (mode == 0 || mode == 3) ? a.p[e] : 0.0f;
+            yv[i] = r < re && mode != 1 ? ld_early(y + e) : 0.0f;
+            pv[i] = r < re && (mode == 0 || mode == 3) ? ld_early(a.p + e) : 0.0f;
         }
     };
     // (done may be stale; the read after the wait decides)

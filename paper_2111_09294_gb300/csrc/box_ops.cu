@@ -279,8 +279,8 @@ __device__ __forceinline__ void prolong_box(const BoxDev<double> &B, int s, int 
     auto load3 = [&](int d) {
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            yv[i] = mode != 1 ? y[d + i] : 0.0;
-            pv[i] = mode == 0 ? p[d + i] : 0.0;
+            yv[i] = mode != 1 ? ld_early(y + d + i) : 0.0;
+            pv[i] = mode == 0 ? ld_early(p + d + i) : 0.0;
         }
     };
     auto load_node = [&]() {
@@ -442,12 +442,12 @@ __device__ __forceinline__ bool restrict_update_unit(const RowBoxDev &B, int uni
         for (int i = 0; i < OWN; ++i) {
             const int r = oBegin + i * T;
             const bool ok = r < oEnd;
-            ro[i] = ok ? r_cur[r] : 0.0f;
-            po[i] = ok && mode == 0 ? p[r] : 0.0f;
-            uo[i] = ok && mode == 0 ? u[r] : 0.0f;
+            ro[i] = ok ? ld_early(r_cur + r) : 0.0f;
+            po[i] = ok && mode == 0 ? ld_early(p + r) : 0.0f;
+            uo[i] = ok && mode == 0 ? ld_early(u + r) : 0.0f;
         }
 #pragma unroll
-        for (int i = 0; i < EXT; ++i) re[i] = ed[i] >= 0 ? (YV ? yv[ed[i]] : r_cur[ed[i]]) : 0.0f;
+        for (int i = 0; i < EXT; ++i) re[i] = ed[i] >= 0 ? ld_early((YV ? yv : r_cur) + ed[i]) : 0.0f;
     };
     // launches queued past a stop load nothing early (a read that may be
     // stale; the one after the wait decides)
@@ -760,8 +760,8 @@ __device__ __forceinline__ void prolong_rows_unit(const RowBoxDev &B, int unit,
 #pragma unroll
             for (int c = 0; c < M; ++c)
                 z[i][c] = ok ? ld_keep(Z + (size_t)c * RO + r, keep) : 0.0f;
-            yv[i] = ok && mode != 1 ? y[r] : 0.0f;
-            pv[i] = ok && mode == 0 ? p[r] : 0.0f;
+            yv[i] = ok && mode != 1 ? ld_early(y + r) : 0.0f;
+            pv[i] = ok && mode == 0 ? ld_early(p + r) : 0.0f;
         }
     };
     const bool early = __ldcg(&sc->done) == kRunning;   // may be stale, as above

@@ -45,6 +45,16 @@ __device__ __forceinline__ int ld_early(const int *a) {
     asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
     return v;
 }
+__device__ __forceinline__ float ld_early(const float *a) {
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ double ld_early(const double *a) {
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(a) : "memory");
+    return v;
+}
 
 // asynchronous 4-byte copy into shared memory with the same policy; a thread
 // that reads back only what it copied itself needs no barrier, just the wait

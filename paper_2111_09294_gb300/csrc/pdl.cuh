@@ -6,10 +6,11 @@
 // touching anything it wrote.  A kernel triggers only after its own wait: so
 // when its successor's blocks run, everything up to the kernel before the
 // predecessor is complete, and the successor may read, before its own wait,
-// set-up data and whatever the predecessor does not write.  That is what the
-// early launch is for: the blocks that fill an SM as it drains load the next
-// kernel's factors, bases and matrix stages meanwhile.  The wait is a no-op
-// for a kernel launched without the attribute.
+// set-up data and, from L2 (ld_early: it is the wait that makes earlier writes
+// visible to ordinary loads), whatever the predecessor does not write.  That
+// is what the early launch is for: the blocks that fill an SM as it drains
+// load the next kernel's factors, bases and matrix stages meanwhile.  The wait
+// is a no-op for a kernel launched without the attribute.
 //
 // Triggers pay where measured: in the FP32 product, the coarse solve and (up
 // to kTriggerBlocks blocks) the prolongation, 31.8 against 35.3 us per FP32

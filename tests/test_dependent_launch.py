@@ -53,3 +53,12 @@ def test_a_held_system_is_not_read_before_the_wait():
     early = re.search(r"const bool early\s*=\s*([^;]*);\s*if \(early\) load_vectors\(\);", text)
     assert early and "ld_early(&bs->go)" in early.group(1)
     assert text.count("load_vectors()") == 1
+
+
+# vectors that an earlier kernel of the run wrote are complete before some waits,
+# but visible to ordinary loads only after them: from L2 there (a thread's own
+# arrays have an index of their own, i, or a size)
+@pytest.mark.parametrize("where", before_wait(), ids=lambda w: f"{w[0]}:{w[1]}")
+def test_vectors_before_the_wait_come_from_l2(where):
+    plain = re.findall(r"(?:(?<![.\w])|\ba\.)(?:r_cur|yv|y|p|u|q|r|x|a|b)\[([^\]]*)\]", where[2])
+    assert not set(plain) - {"i", "R", "3"}, where[:2]

@@ -156,8 +156,8 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
     constexpr int LPS = MB / 4, SPP = 32 / LPS;   // lanes per slot, slots per pass
     const SpmvDev<float> &A = args.A;
     const int m = args.m, fin = args.fin;
-    const float *__restrict__ x = args.x;
-    const float *__restrict__ b = args.b;
+    const float *x = args.x;
+    const float *b = args.b;
     float *__restrict__ y = args.y;
     BatchScalars *bs = args.bs;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -257,7 +257,7 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const size_t at = ((size_t)row * 3 + i) * LPS + qc;
-            const float4 s4 = reinterpret_cast<const float4 *>(RES ? b : x)[at];
+            const float4 s4 = ld_dep(reinterpret_cast<const float4 *>(RES ? b : x) + at);
             float4 o4;
             if (RES) {
                 o4 = make_float4(s4.x - a[0][i][0], s4.y - a[0][i][1], s4.z - a[0][i][2],
@@ -303,7 +303,7 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
         const int c = reinterpret_cast<const int *>(ring + st * SB)[t * 32 + q * SPP + sl0];
         const float4 *xc = reinterpret_cast<const float4 *>(x) + (size_t)c * (3 * LPS) + qc;
 #pragma unroll
-        for (int jc = 0; jc < 3; ++jc) xv[jc] = __ldg(xc + jc * LPS);
+        for (int jc = 0; jc < 3; ++jc) xv[jc] = ld_dep(xc + jc * LPS);
     };
     int sS, cP, curN = 0, cslot = 0, consumed = 0;
     uint32_t cpar = 0u;
@@ -831,7 +831,7 @@ __device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int
             if (V == 4) {
                 if (4 * lane < clen) {
                     const float4 v =
-                        __ldg(reinterpret_cast<const float4 *>(g0 + (size_t)j * a.gld + 4 * lane));
+                        ld_dep(reinterpret_cast<const float4 *>(g0 + (size_t)j * a.gld + 4 * lane));
                     g[0] = v.x;
                     g[1] = v.y;
                     g[2] = v.z;
@@ -840,7 +840,7 @@ __device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int
             } else {
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    if (lane + 32 * q < clen) g[q] = __ldg(g0 + (size_t)j * a.gld + lane + 32 * q);
+                    if (lane + 32 * q < clen) g[q] = ld_dep(g0 + (size_t)j * a.gld + lane + 32 * q);
             }
 #pragma unroll
             for (int r = 0; r < RB; ++r) {

@@ -5,6 +5,7 @@
 // one dense product per block.  The FP32 path applies the inverse of the
 // block-scaled system's blocks, L_b^T (K_bb)^-1 L_b (L the node-block Cholesky
 // factors that scale K~ = L^-1 K L^-T), rounded to FP32.
+#include "cache.cuh"
 #include "factor.cuh"
 #include "reduce.cuh"
 
@@ -115,7 +116,7 @@ void launch_scale_block_inverse(int n, const int *rowBlock, const int *bStart, c
 // to 1,740 dofs (24^3, FP32 solve): 3.96 ms before, 3.63 now.
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-k_block_apply(BlkDev<T> B, const T *__restrict__ r, T *__restrict__ y, double *partials,
+k_block_apply(BlkDev<T> B, const T *r, T *__restrict__ y, double *partials,
               Scalars *sc) {
     constexpr int R = 4;
     __shared__ T rs[XDCG_MAX_BLOCK_DOFS];
@@ -141,7 +142,7 @@ k_block_apply(BlkDev<T> B, const T *__restrict__ r, T *__restrict__ y, double *p
     if (early && iFirst < i1 && lane + 96 < nb) load(iFirst, lane);
     pdl_wait();
     if (sc->done != kRunning) return;
-    for (int j = threadIdx.x; j < nb; j += blockDim.x) rs[j] = r[B.idx[p0 + j]];
+    for (int j = threadIdx.x; j < nb; j += blockDim.x) rs[j] = ld_dep(r + B.idx[p0 + j]);
     __syncthreads();
     T part = T(0);
     for (int i = iFirst; i < i1; i += R * kWarps) {

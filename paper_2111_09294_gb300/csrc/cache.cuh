@@ -56,6 +56,35 @@ __device__ __forceinline__ double ld_early(const double *a) {
     return v;
 }
 
+// What an earlier kernel of the run wrote, read after the wait: the ordinary
+// path through L1.  The read-only path (__ldg, or what the compiler makes of a
+// const __restrict__ pointer) is for data that nothing writes while the kernel
+// is resident, and a kernel launched early is resident while the one before it
+// still writes; nor is such a load held behind the wait.  (No memory clobber: a
+// kernel does not write what it reads so.)
+__device__ __forceinline__ float ld_dep(const float *a) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(a));
+    return v;
+}
+__device__ __forceinline__ double ld_dep(const double *a) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(a));
+    return v;
+}
+__device__ __forceinline__ float4 ld_dep(const float4 *a) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(a));
+    return v;
+}
+__device__ __forceinline__ double2 ld_dep(const double2 *a) {
+    double2 v;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(a));
+    return v;
+}
+
 // asynchronous 4-byte copy into shared memory with the same policy; a thread
 // that reads back only what it copied itself needs no barrier, just the wait
 __device__ __forceinline__ void cp_keep(float *smem, const float *a, uint64_t pol) {

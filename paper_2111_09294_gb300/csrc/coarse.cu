@@ -243,8 +243,8 @@ __device__ __forceinline__ void coarse_scalars(double blk, int rowBlk, int mode,
 // recursive one it replaced (kept in scratch[3]): the recursion had drifted
 // too far from the true residual for the old direction to stay conjugate.
 __global__ void __launch_bounds__(kThreads)
-k_coarse(const double *__restrict__ Einv, int k, const double *__restrict__ g,
-         const double *__restrict__ zr, double *nu, float *nu32, int mode, double *partials,
+k_coarse(const double *__restrict__ Einv, int k, const double *g,
+         const double *zr, double *nu, float *nu32, int mode, double *partials,
          ResidualSums sums, Scalars *sc) {
     pdl_wait();
     if (sc->done != kRunning) return;
@@ -262,24 +262,24 @@ k_coarse(const double *__restrict__ Einv, int k, const double *__restrict__ g,
             int j = lane;
             for (; j + 32 < k2; j += 64) {
                 const double2 a = __ldg(r2 + j), b = __ldg(r2 + j + 32);
-                const double2 x = __ldg(g2 + j), y = __ldg(g2 + j + 32);
+                const double2 x = ld_dep(g2 + j), y = ld_dep(g2 + j + 32);
                 s0 = fma(a.x, x.x, s0);
                 s1 = fma(a.y, x.y, s1);
                 s2 = fma(b.x, y.x, s2);
                 s3 = fma(b.y, y.y, s3);
             }
             for (; j < k2; j += 32) {
-                const double2 a = __ldg(r2 + j), x = __ldg(g2 + j);
+                const double2 a = __ldg(r2 + j), x = ld_dep(g2 + j);
                 s0 = fma(a.x, x.x, s0);
                 s1 = fma(a.y, x.y, s1);
             }
         } else {
             int j = lane;
             for (; j + 32 < k; j += 64) {
-                s0 = fma(__ldg(row + j), __ldg(g + j), s0);
-                s1 = fma(__ldg(row + j + 32), __ldg(g + j + 32), s1);
+                s0 = fma(__ldg(row + j), ld_dep(g + j), s0);
+                s1 = fma(__ldg(row + j + 32), ld_dep(g + j + 32), s1);
             }
-            for (; j < k; j += 32) s0 = fma(__ldg(row + j), __ldg(g + j), s0);
+            for (; j < k; j += 32) s0 = fma(__ldg(row + j), ld_dep(g + j), s0);
         }
         double s = (s0 + s1) + (s2 + s3);
 #pragma unroll
@@ -320,8 +320,8 @@ constexpr int kCoarse32Rows = 4, kCoarse32Threads = 64;
 
 template <int V>
 __global__ void __launch_bounds__(kCoarse32Threads)
-k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
-           const double *__restrict__ zr, double *nu, float *nu32, int mode, double *partials,
+k_coarse32(const float *__restrict__ Einv, int k, const float *g32,
+           const double *zr, double *nu, float *nu32, int mode, double *partials,
            ResidualSums sums, Scalars *sc) {
     constexpr int R = kCoarse32Rows, U = V == 4 ? 4 : 8;
     using E = typename std::conditional<V == 4, float4, float>::type;
@@ -362,7 +362,7 @@ k_coarse32(const float *__restrict__ Einv, int k, const float *__restrict__ g32,
         E x[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j + 32 * u < j1) x[u] = __ldg(gv + j + 32 * u);
+            if (j + 32 * u < j1) x[u] = ld_dep(gv + j + 32 * u);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (j + 32 * u < j1) {

@@ -8,6 +8,7 @@
 // evict-first loads; the gathered x chunks stay in L1/L2.
 #include <algorithm>
 
+#include "cache.cuh"
 #include "reduce.cuh"
 #include "spmv_cfg.cuh"
 #include "tma.cuh"
@@ -43,7 +44,7 @@ namespace xdcg {
 // 32^3 (416 groups) 9.34 both.
 template <typename T, bool RES, int SHAPE, int W>
 __global__ void __launch_bounds__(32 * W, SpmvCfg<T, SHAPE>::MINB * (kSpmvWarps / W))
-k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__restrict__ b,
+k_spmv(SpmvDev<T> A, const T *x, T *__restrict__ y, const T *b,
        double *partials, Scalars *sc, int fin, int slot, SpmvCols cols) {
     using Cfg = SpmvCfg<T, SHAPE>;
     if (cols.list) {   // several columns in one launch: blockIdx.y picks this block's
@@ -154,9 +155,9 @@ k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__rest
     auto fetch_row_entries = [&]() {
         pend = false;
         if (own) {
-            e0 = ev[r3];
-            e1 = ev[r3 + 1];
-            e2 = ev[r3 + 2];
+            e0 = ld_dep(ev + r3);
+            e1 = ld_dep(ev + r3 + 1);
+            e2 = ld_dep(ev + r3 + 2);
         }
     };
     auto finish = [&]() {
@@ -187,9 +188,9 @@ k_spmv(SpmvDev<T> A, const T *__restrict__ x, T *__restrict__ y, const T *__rest
         for (int t = 0; t < C; ++t) {
             if (t < n) {
                 const int c = cs[t * 32 + lane];
-                xv[t][0] = __ldg(x + 3 * c);
-                xv[t][1] = __ldg(x + 3 * c + 1);
-                xv[t][2] = __ldg(x + 3 * c + 2);
+                xv[t][0] = ld_dep(x + 3 * c);
+                xv[t][1] = ld_dep(x + 3 * c + 1);
+                xv[t][2] = ld_dep(x + 3 * c + 2);
             }
         }
     };
@@ -328,8 +329,8 @@ struct LeanWalk {
 // stage loop is unrolled by two).
 template <bool RES, int SHAPE>
 __global__ void __launch_bounds__(kSpmvThreads, SpmvCfg<float, SHAPE>::MINB)
-k_spmv_lean(SpmvDev<float> A, const float *__restrict__ x, float *__restrict__ y,
-            const float *__restrict__ b, double *partials, Scalars *sc, int fin, int slot) {
+k_spmv_lean(SpmvDev<float> A, const float *x, float *__restrict__ y, const float *b,
+            double *partials, Scalars *sc, int fin, int slot) {
     using Cfg = SpmvCfg<float, SHAPE>;
     constexpr int C = Cfg::C, NS = Cfg::NS, SB = stage_bytes<float, SHAPE>();
     extern __shared__ __align__(128) unsigned char smem[];
@@ -421,9 +422,9 @@ k_spmv_lean(SpmvDev<float> A, const float *__restrict__ x, float *__restrict__ y
     auto fetch_row_entries = [&]() {
         pend = false;
         if (own) {
-            e0 = ev[r3];
-            e1 = ev[r3 + 1];
-            e2 = ev[r3 + 2];
+            e0 = ld_dep(ev + r3);
+            e1 = ld_dep(ev + r3 + 1);
+            e2 = ld_dep(ev + r3 + 2);
         }
     };
     auto finish = [&]() {
@@ -474,9 +475,9 @@ k_spmv_lean(SpmvDev<float> A, const float *__restrict__ x, float *__restrict__ y
         for (int t = 0; t < C; ++t) {
             if (t < n) {
                 const int c = cs[t * 32 + lane];
-                xv[t][0] = __ldg(x + 3 * c);
-                xv[t][1] = __ldg(x + 3 * c + 1);
-                xv[t][2] = __ldg(x + 3 * c + 2);
+                xv[t][0] = ld_dep(x + 3 * c);
+                xv[t][1] = ld_dep(x + 3 * c + 1);
+                xv[t][2] = ld_dep(x + 3 * c + 2);
             }
         }
     };

@@ -62,3 +62,22 @@ def test_a_held_system_is_not_read_before_the_wait():
 def test_vectors_before_the_wait_come_from_l2(where):
     plain = re.findall(r"(?:(?<![.\w])|\ba\.)(?:r_cur|yv|y|p|u|q|r|x|a|b)\[([^\]]*)\]", where[2])
     assert not set(plain) - {"i", "R", "3"}, where[:2]
+
+
+# set-up data, complete before any kernel of a run: the tables and their offsets,
+# E^-1, the restriction's records and its blocks of W
+SETUP = {"off", "off + mid", "off + s", "off + s + 1", "tab", "Einv", "r2 + j", "r2 + j + 32",
+         "row + j", "row + j + 32", "B.ext.rec + e0 + ch0 * CE + i",
+         "B.own.rec + z0 + ch0 * CO + i", "b + i * M"}
+
+
+def test_read_only_loads_are_of_setup_data():
+    waiting = {n for _, n, _ in before_wait()} | {"k_spmm_sys", "k_restrict_b_sys", "load",
+                                                  "k_coarse_b_sys", "k_prolong_b_sys", "sys_of"}
+    for f, n, params, body in functions():
+        for arg in re.findall(r"__ldg\(((?:[^()]|\([^()]*\))*)\)", body):
+            assert arg in SETUP, (f, n, arg)
+        if n in waiting:
+            # what is only written (y) may be told apart from the rest
+            for const, name in re.findall(r"(const )?[\w<>]+ \*__restrict__ (\w+)", params + body):
+                assert not const or name in SETUP, (f, n, name)

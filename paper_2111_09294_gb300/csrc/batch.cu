@@ -254,10 +254,16 @@ __device__ __forceinline__ void spmm_body(const SpmmArgs &args, int blk, int nbl
 #pragma unroll
                 for (int j = 0; j < 4; ++j) a[0][i][j] += a[LPS - 1][i][j];
         if (row < 0) return;
+        // loads before the stores, behind which they would wait for one another
+        float4 src[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            src[i] = ld_dep(reinterpret_cast<const float4 *>(RES ? b : x) +
+                            ((size_t)row * 3 + i) * LPS + qc);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const size_t at = ((size_t)row * 3 + i) * LPS + qc;
-            const float4 s4 = ld_dep(reinterpret_cast<const float4 *>(RES ? b : x) + at);
+            const float4 s4 = src[i];
             float4 o4;
             if (RES) {
                 o4 = make_float4(s4.x - a[0][i][0], s4.y - a[0][i][1], s4.z - a[0][i][2],
@@ -930,12 +936,12 @@ void launch_coarse_b(const CoarseBArgs &a, cudaStream_t st) {
 // mode 1 (start): p = Z~ nu; mode 2 (start): p = y + Z~ nu.  y is the current
 // residual buffer.
 //
-// A thread's rows are all in flight at once: their rows of Z~, and in an
-// iteration that runs the system their entries of y and p, before the wait for
-// the coarse solve.  No kernel still running writes those, nor the count that
-// picks y's buffer; but in a launch over several systems a held system's
-// replacement, on a stream of its own, writes all three, so the gate's go
-// decides first.  8 columns at 32^3: 9.4 us before, 9.2 now.
+// A thread's rows are all in flight at once: their rows of Z~ before the wait
+// for the coarse solve, their entries of y and p after it, beside those of nu.
+// (Not before: in a launch over several systems a held system's replacement, on
+// a stream of its own, writes both, and the count that picks y's buffer; 8
+// columns at 32^3: 9.2 us, 9.0 with both before the wait, and 16.4 with every
+// warp asking L2 first whether the system is held.)
 template <int MB, int M>
 __device__ __forceinline__ void prolong_b_unit(const ProlongBArgs &a, int unit) {
     constexpr int kRowStep = kThreads / MB, R = (kProlongRowsBatch + kRowStep - 1) / kRowStep;
@@ -955,20 +961,6 @@ __device__ __forceinline__ void prolong_b_unit(const ProlongBArgs &a, int unit) 
         for (int c = 0; c < M; ++c)
             z[i][c] = r < re ? ld_keep(Z + (size_t)c * RO + r, keep) : 0.0f;
     }
-    auto load_vectors = [&]() {
-        const float *y = (ld_early(&bs->its) & 1) ? a.rB : a.rA;
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-            const int r = rb + i * kRowStep;
-            const size_t e = (size_t)r * MB + j;
-            yv[i] = r < re && mode != 1 ? ld_early(y + e) : 0.0f;
-            pv[i] = r < re && (mode == 0 || mode == 3) ? ld_early(a.p + e) : 0.0f;
-        }
-    };
-    // (done may be stale; the read after the wait decides)
-    const bool early =
-        mode == 0 && ld_early(&bs->go) != 0 && ld_early(&bs->done) == kRunning;
-    if (early) load_vectors();
     pdl_wait();
     if (!batch_runs(bs, mode == 0)) return;
     bool leaves = false;
@@ -978,7 +970,14 @@ __device__ __forceinline__ void prolong_b_unit(const ProlongBArgs &a, int unit) 
         if (j >= a.m || !bs->repl[j]) return;
         leaves = !bs->active[j];
     }
-    if (!early) load_vectors();
+    const float *y = (bs->its & 1) ? a.rB : a.rA;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int r = rb + i * kRowStep;
+        const size_t e = (size_t)r * MB + j;
+        yv[i] = r < re && mode != 1 ? y[e] : 0.0f;
+        pv[i] = r < re && (mode == 0 || mode == 3) ? a.p[e] : 0.0f;
+    }
     const float beta = (mode == 0 || mode == 3) && !leaves ? (float)bs->beta[j] : 0.0f;
     float nv[M];
 #pragma unroll

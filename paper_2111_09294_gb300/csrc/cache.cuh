@@ -40,19 +40,9 @@ __device__ __forceinline__ float4 ld_keep(const float4 *a, uint64_t pol) {
 // not set-up data: from L2, where everything that a finished kernel wrote is.
 // A plain load might find an older line in the SM's L1, since the wait, which
 // makes earlier writes visible, has yet to come.  Not moved across the wait.
-__device__ __forceinline__ int ld_early(const int *a) {
-    int v;
-    asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
-    return v;
-}
 __device__ __forceinline__ float ld_early(const float *a) {
     float v;
     asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ double ld_early(const double *a) {
-    double v;
-    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(a) : "memory");
     return v;
 }
 

@@ -351,8 +351,11 @@ cudaError_t launch_dense_inverse(const DenseBatch &B, int maxDim, long long nEnt
     if (B.nMat == 0) return cudaSuccess;
     const int smem = 2 * kNB * kLd * (int)sizeof(double);
     // a pivot CTA that fills an SM's shared memory beside no other, while the
-    // matrices leave most SMs to the tiles
-    const int pivotSmem = B.nMat <= 16 ? 190 * 1024 : 0;
+    // matrices leave most SMs to the tiles (measured for one matrix; the line is
+    // a tenth of the SMs).  The limit is the kernel's, for every context and
+    // thread, so it is always the same; only the launch's own size varies
+    constexpr int kPivotSmem = 190 * 1024;
+    const int pivotSmem = B.nMat <= 16 ? kPivotSmem : 0;
     for (auto k : {k_inv_panel, k_inv_update_next}) {
         const cudaError_t e =
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -361,7 +364,7 @@ cudaError_t launch_dense_inverse(const DenseBatch &B, int maxDim, long long nEnt
     cudaError_t e = cudaFuncSetAttribute(k_inv_update_rest,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_inv_pivot, cudaFuncAttributeMaxDynamicSharedMemorySize, pivotSmem);
+    e = cudaFuncSetAttribute(k_inv_pivot, cudaFuncAttributeMaxDynamicSharedMemorySize, kPivotSmem);
     if (e != cudaSuccess) return e;
     k_inv_thresholds<<<B.nMat, kInvThreads, 0, st>>>(B, rel);
     const int steps = (maxDim + kNB - 1) / kNB;

@@ -347,8 +347,8 @@ struct RunFollower {
     bool take(int it) {
         const unsigned long long v = __atomic_load_n(&c->h_prog->rr[it % kRing], __ATOMIC_ACQUIRE);
         if (v == kNoReport) return false;
-        stopped = (v >> 63) != 0;
-        const unsigned long long a = v & 0x7fffffffffffffffull;
+        stopped = (v & kStopBit) != 0;
+        const unsigned long long a = v & ~kStopBit;
         std::memcpy(&rr, &a, sizeof(rr));
         seen = it;
         return true;

@@ -31,11 +31,19 @@ enum Fin : int {
 // flag) is written before that.  A slot holds kNoReport until then: one 8-byte
 // store per iteration, no copy and no event in the stream.
 constexpr int kRing = 64;
-constexpr unsigned long long kNoReport = 0x7ff8dead00000000ull;   // a NaN no sum of squares gives
+constexpr unsigned long long kNoReport = 0x7ff8dead00000000ull;   // a NaN that is never reported
+constexpr unsigned long long kStopBit = 0x8000000000000000ull;
 struct Progress {
     unsigned long long rr[kRing];
     unsigned long long stop;   // its << 32 | done
 };
+// A report of ||r||^2 (its bits): the sign bit says stopped and nothing else, so
+// a NaN, whose sign and payload may be anything, is reported as one fixed NaN.
+__host__ __device__ inline unsigned long long report_word(unsigned long long rr, bool stopped) {
+    rr &= ~kStopBit;
+    if (rr > 0x7ff0000000000000ull) rr = 0x7ff8000000000000ull;
+    return stopped ? rr | kStopBit : rr;
+}
 
 // Scalars of one CG run, in device memory.  Written only by the last block
 // of a reduction kernel (single writer), read by all later kernels.

@@ -407,15 +407,15 @@ __device__ __forceinline__ bool last_block(unsigned int *ticket) {
 __device__ __forceinline__ void report(const Scalars *sc) {
     volatile Progress *p = sc->prog;
     if (!p) return;
-    unsigned long long v = (unsigned long long)__double_as_longlong(sc->rr);
-    if (sc->done == kRunning) {
+    const bool stopped = sc->done != kRunning;
+    if (!stopped) {
         if (sc->rr == 0.0) return;   // a prolongation before the first residual
     } else {
         p->stop = (unsigned long long)(unsigned int)sc->its << 32 | (unsigned int)sc->done;
         __threadfence_system();
-        v |= 0x8000000000000000ull;
     }
-    p->rr[sc->its % kRing] = v;
+    p->rr[sc->its % kRing] =
+        report_word((unsigned long long)__double_as_longlong(sc->rr), stopped);
 }
 
 // Shared last-block actions on the scalar block.  FinLoads: what they read,

@@ -225,9 +225,7 @@ k_update_plain(T *u, T *r, const T *p, const T *q, long long n, int mode, double
         v[0] = fma(ri, ri, v[0]);
     }
     double tot;
-    FinLoads in;
-    if (grid_sum<T>(v[0], partials, &sc->ticket[2], tot, [&] { in.load(sc); }) &&
-        threadIdx.x == 0) {
+    if (grid_sum<T>(v[0], partials, &sc->ticket[2], tot, [] {}) && threadIdx.x == 0) {
         sc->rr = tot;
         if (sc->hist && sc->its < sc->histCap) sc->hist[sc->its] = tot;
         if (tot <= sc->tol2ff)

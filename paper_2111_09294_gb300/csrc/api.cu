@@ -329,11 +329,15 @@ xdcg_status phase_collect(xdcg_ctx *c, int n, int P, xdcg_result *res) {
     } while (0)
 
 // Follows a run by its reports (Progress).  The host enqueues the next kUnitIts
-// iterations when kAheadIts are left past the last one reported: the device
-// never waits for it, at most kAheadIts + kUnitIts - 1 iterations are queued
-// past a stop (four or five launches of ~2 us each; 8 to 16 with a stream copy
-// and an event per 8 iterations before), and nothing is read back through the
-// stream.  Per FP32 iteration 12^3 31.8 -> 27.2 us, 48^3 84.7 -> 78.0 us.
+// iterations when kAheadIts are left past the last one reported: at most
+// kAheadIts + kUnitIts - 1 iterations are queued past a stop (four or five
+// launches of ~2 us each; 8 to 16 with a stream copy and an event per 8
+// iterations before), and nothing is read back through the stream.  Per FP32
+// iteration 12^3 31.8 -> 27.2 us, 48^3 84.7 -> 78.0 us.  The two iterations left
+// (50 us at 8^3) cover the enqueuing of four while each solving host thread has
+// a core: 8 threads make 3,777 mixed solves at 8^3 a second, 3,261 with 8 to 16
+// iterations ahead.  The thread spins all the while; threads that share a core
+// take turns (two on one core: the throughput of one).
 struct RunFollower {
     xdcg_ctx *c;
     int seen;                     // the last iteration reported
@@ -580,23 +584,20 @@ void coarse_inner(xdcg_ctx *c, const double *zr, int mode, Scalars *sc, cudaStre
 void scaled_init(xdcg_ctx *c, const float *f, float *u, float *rA, float *p, Scalars *sc) {
     cudaStream_t st = c->st;
     Level32 &L = c->L32;
-    launch_restrict_update(L.R, nullptr, f, nullptr, nullptr, nullptr, 2, c->g, nullptr,
-                           c->partials, sc, st);
+    launch_restrict_start(L.R, f, 2, c->g, nullptr, c->partials, sc, st);
     coarse_inner(c, nullptr, 0, sc, st);
     launch_prolong_rows(L.R, c->nu32, nullptr, u, 1, sc, st);
     launch_spmv<float>(L.A, u, rA, f, 1, c->partials, sc, kFinRR, 0, st);
     if (c->userBlocks) {
         // y = M~^-1 r by the caller blocks, then g = Z~^T r - W~^T y
         launch_block_apply<float>(L.J, rA, c->y32, c->partials, sc, st);
-        launch_restrict_update(L.R, nullptr, rA, nullptr, nullptr, nullptr, 3, c->g, c->zr,
-                               c->partials, sc, st, c->y32);
+        launch_restrict_start(L.R, rA, 3, c->g, c->zr, c->partials, sc, st, c->y32);
         coarse_inner(c, c->zr, 1, sc, st);
         launch_prolong_rows(L.R, c->nu32, c->y32, p, 2, sc, st);
         c->launches += 8;
         return;
     }
-    launch_restrict_update(L.R, nullptr, rA, nullptr, nullptr, nullptr, 1, c->g, c->zr,
-                           c->partials, sc, st);
+    launch_restrict_start(L.R, rA, 1, c->g, c->zr, c->partials, sc, st);
     coarse_inner(c, c->zr, 1, sc, st);
     launch_prolong_rows(L.R, c->nu32, rA, p, 2, sc, st);
     c->launches += 7;
@@ -645,12 +646,11 @@ xdcg_status scaled_iterate(xdcg_ctx *c, float *u, float *rA, float *rB, float *p
                 // = M~^-1 r by the caller blocks, then the restriction
                 launch_update_plain<float>(u, rA, p, q, c->n, 0, c->partials, sc, s);
                 launch_block_apply<float>(L.J, rA, c->y32, c->partials, sc, s);
-                launch_restrict_update(L.R, nullptr, rA, nullptr, nullptr, nullptr, 3, c->g, c->zr,
-                                       c->partials, sc, s, c->y32);
+                launch_restrict_start(L.R, rA, 3, c->g, c->zr, c->partials, sc, s, c->y32);
                 c->launches += 2;
             } else {
-                launch_restrict_update_deferred(L.R, u, rc, rn, p, q, c->g, c->zr, rrPart, sc, pqPart,
-                                                L.A.grid, s);
+                launch_restrict_update(L.R, u, rc, rn, p, q, c->g, c->zr, rrPart, sc, pqPart,
+                                       L.A.grid, s);
             }
         } else if (m == 2) {
             coarse_inner(c, c->zr, 2, sc, s, ResidualSums{rrPart, L.R.nUnits, 1});
@@ -888,12 +888,10 @@ xdcg_status solve_mixed(xdcg_ctx *c, const double *f, double *u, double tol, boo
             launch_update_plain<float>(nullptr, rbuf, nullptr, nullptr, c->n, 1, c->partials,
                                        c->sc32, st);
             launch_block_apply<float>(L.J, rbuf, c->y32, c->partials, c->sc32, st);
-            launch_restrict_update(L.R, nullptr, rbuf, nullptr, nullptr, nullptr, 3, c->g, c->zr,
-                                   c->partials, c->sc32, st, c->y32);
+            launch_restrict_start(L.R, rbuf, 3, c->g, c->zr, c->partials, c->sc32, st, c->y32);
             c->launches += 2;
         } else {
-            launch_restrict_update(L.R, nullptr, rbuf, nullptr, nullptr, nullptr, 1, c->g, c->zr,
-                                   c->partials, c->sc32, st);
+            launch_restrict_start(L.R, rbuf, 1, c->g, c->zr, c->partials, c->sc32, st);
         }
         coarse_inner(c, c->zr, done == kBreakdown ? 1 : 3, c->sc32, st);
         launch_prolong_rows(L.R, c->nu32, c->userBlocks ? c->y32 : rbuf, c->p32,

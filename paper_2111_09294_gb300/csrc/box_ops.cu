@@ -16,7 +16,7 @@ namespace xdcg {
 
 // ---- restriction (FP64) ------------------------------------------------------
 //
-// One CTA per six coarse columns of a box (RestrictUnit), the units with the
+// One CTA per six coarse columns of a box (BoxDev::unit), the units with the
 // most rows first.  The lanes of a warp form five groups of six lanes; lane
 // (group, column c) accumulates column c over every slots-th node of the box
 // (box_slots), so every lane keeps one running sum and the only cross-lane
@@ -614,13 +614,13 @@ __device__ __forceinline__ bool restrict_update_unit(const RowBoxDev &B, int uni
     return true;
 }
 
-// Deferred form (deferred != 0, mode 0 of an iteration of the FP32 iteration): the
-// product left its blocks' sums of p^T q in pqPart instead of reducing them
-// itself; every block adds them (block_total_t0), takes alpha = rho / pq,
-// and block 0 records pq, alpha and counts the iteration (its += 1: the
-// launch's arguments do not depend on the iteration, so a captured batch of
-// iterations can be replayed), or the breakdown (or a failed wait of the
-// product).  Its blocks' sums of ||r||^2 stay in partials, for the coarse solve.
+// Mode 0 (an iteration): the product left its blocks' sums of p^T q in pqPart
+// instead of reducing them itself; every block adds them (block_total_t0), takes
+// alpha = rho / pq, and block 0 records pq, alpha and counts the iteration (its
+// += 1: the launch's arguments do not depend on the iteration, so a captured
+// batch of iterations can be replayed), or the breakdown (or a failed wait of
+// the product).  Its blocks' sums of ||r||^2 stay in partials, for the coarse
+// solve; mode 1 (start, replacement) adds them itself.
 //
 // Bound by latency: 51 MB at 48^3, most of it from L2, between two grid-wide
 // dependencies.  48^3 (543 units): 28.8 us before (dependent loads after the
@@ -630,16 +630,13 @@ template <bool YV, bool FEW>
 __global__ void __launch_bounds__(kRowThreads, FEW ? 1 : 4)
 k_restrict_update(RowBoxDev B, float *u, const float *r_cur, float *r_next, const float *p,
                   const float *q, const float *yv, int mode, double *g, double *zr,
-                  double *partials, Scalars *sc, int deferred, const float2 *pqPart, int pqN) {
+                  double *partials, Scalars *sc, const float2 *pqPart, int pqN) {
     extern __shared__ __align__(16) float stage[];
     __shared__ float red[8][32];
     const int unit = blockIdx.x;
     // after the wait: alpha, the same for every thread; false: nothing to do
     auto alpha_of = [&](float &alpha) -> bool {
-        if (!deferred) {
-            alpha = (mode == 0) ? (float)sc->alpha : 0.0f;
-            return true;
-        }
+        if (mode != 0) return true;   // no update: alpha stays 0
         __shared__ float sAlpha;
         __shared__ bool sGo;
         const double pq = block_total_t0(pqPart, pqN);
@@ -674,11 +671,8 @@ k_restrict_update(RowBoxDev B, float *u, const float *r_cur, float *r_next, cons
             : restrict_update_unit<6, YV, FEW>(B, unit, u, r_cur, r_next, p, q, yv, mode, g, zr,
                                                sc, stage, red, alpha_of, rr);
     if (!went || mode >= 2) return;
-    if (deferred) {
-        if (threadIdx.x == 0) partials[blockIdx.x] = (double)rr;
-        return;
-    }
     if (threadIdx.x == 0) partials[blockIdx.x] = (double)rr;
+    if (mode == 0) return;
     if (!last_block(&sc->ticket[2])) return;
     const double tot = sum_slots<kRowThreads>(partials, (int)gridDim.x);
     if (threadIdx.x == 0) {
@@ -697,10 +691,10 @@ template <bool YV, bool FEW>
 static void launch_restrict_rows(const RowBoxDev &B, float *u, const float *r_cur, float *r_next,
                                  const float *p, const float *q, const float *y, int mode,
                                  double *g, double *zr, double *partials, Scalars *sc,
-                                 int deferred, const float2 *pqPart, int pqN, cudaStream_t st) {
+                                 const float2 *pqPart, int pqN, cudaStream_t st) {
     launch_pdl(k_restrict_update<YV, FEW>, B.nUnits, kRowThreads,
                kStageFloats<FEW> * kRowThreads * sizeof(float), st, B, u, r_cur, r_next, p, q, y,
-               mode, g, zr, partials, sc, deferred, pqPart, pqN);
+               mode, g, zr, partials, sc, pqPart, pqN);
 }
 
 // dynamic shared memory of the restriction's staging (once per context)
@@ -716,29 +710,28 @@ bool restrict_rows_prepare() {
 }
 
 // FEW when every unit has an SM to itself
-void launch_restrict_update(const RowBoxDev &B, float *u, const float *r_cur, float *r_next,
-                            const float *p, const float *q, int mode, double *g, double *zr,
-                            double *partials, Scalars *sc, cudaStream_t st, const float *y) {
+void launch_restrict_start(const RowBoxDev &B, const float *r, int mode, double *g, double *zr,
+                           double *partials, Scalars *sc, cudaStream_t st, const float *y) {
     const bool few = B.nUnits <= device_sm_count();
     auto launch = mode == 3 ? (few ? launch_restrict_rows<true, true> : launch_restrict_rows<true, false>)
                             : (few ? launch_restrict_rows<false, true> : launch_restrict_rows<false, false>);
-    launch(B, u, r_cur, r_next, p, q, y, mode, g, zr, partials, sc, 0, nullptr, 0, st);
+    launch(B, nullptr, r, nullptr, nullptr, nullptr, y, mode, g, zr, partials, sc, nullptr, 0, st);
 }
 
-void launch_restrict_update_deferred(const RowBoxDev &B, float *u, const float *r_cur,
-                                     float *r_next, const float *p, const float *q, double *g,
-                                     double *zr, double *rrPart, Scalars *sc,
-                                     const float2 *pqPart, int pqN, cudaStream_t st) {
+void launch_restrict_update(const RowBoxDev &B, float *u, const float *r_cur, float *r_next,
+                            const float *p, const float *q, double *g, double *zr,
+                            double *rrPart, Scalars *sc, const float2 *pqPart, int pqN,
+                            cudaStream_t st) {
     auto launch = B.nUnits <= device_sm_count() ? launch_restrict_rows<false, true>
                                                 : launch_restrict_rows<false, false>;
-    launch(B, u, r_cur, r_next, p, q, nullptr, 0, g, zr, rrPart, sc, 1, pqPart, pqN, st);
+    launch(B, u, r_cur, r_next, p, q, nullptr, 0, g, zr, rrPart, sc, pqPart, pqN, st);
 }
 
 // Triggers its dependent, the next product, only while its grid is small: the
 // product's blocks fill the SMs as they are, and a large prolongation finishes
 // later beside them (32^3, 512 blocks: 46.3 us per iteration with, 47.0
-// without; 48^3, 1,066 blocks: 79.4 and 78.0).
-constexpr int kTriggerBlocks = 608;   // four per SM
+// without; 48^3, 1,066 blocks: 79.4 and 78.0; nothing was measured between).
+constexpr int kTriggerBlocks = 608;   // four for each of 152 SMs
 
 // Prolongation over one unit's own rows, kProlongRows / kRowThreads rows a
 // thread, all in flight before the wait for the coarse solve: their rows of

@@ -267,34 +267,32 @@ void launch_restrict(const BoxDev<double> &B, const double *a, const double *b, 
                      double *g, double *zr, const Scalars *sc, cudaStream_t st);
 void launch_prolong(const BoxDev<double> &B, const double *nu, const double *y, double *p,
                     int mode, Scalars *sc, cudaStream_t st);
-// mode 0 (iteration): r' = r - alpha q and u += alpha p on own rows (r' written
-// to r_next), g = Z~^T r' - W~^T r', zr = Z~^T r', ||r'||^2 with the
-// convergence and iteration-cap tests; mode 1 (start): the same without the
-// update (alpha = 0, nothing written but g, zr, ||r||^2); mode 2 (Algorithm
-// 2): g = Z~^T r only; mode 3 (caller blocks, y = M~^-1 r given): g = Z~^T r
-// - W~^T y and zr = Z~^T r, nothing else.
-void launch_restrict_update(const RowBoxDev &B, float *u, const float *r_cur, float *r_next,
-                            const float *p, const float *q, int mode, double *g, double *zr,
-                            double *partials, Scalars *sc, cudaStream_t st,
-                            const float *y = nullptr);
+// mode 1 (start, or a replaced residual): g = Z~^T r - W~^T r, zr = Z~^T r,
+// ||r||^2 with the convergence and iteration-cap tests; mode 2 (Algorithm 2):
+// g = Z~^T r only; mode 3 (caller blocks, y = M~^-1 r given): g = Z~^T r -
+// W~^T y and zr = Z~^T r, nothing else.
+void launch_restrict_start(const RowBoxDev &B, const float *r, int mode, double *g, double *zr,
+                           double *partials, Scalars *sc, cudaStream_t st,
+                           const float *y = nullptr);
 bool restrict_rows_prepare();
 void launch_prolong_rows(const RowBoxDev &B, const float *nu32, const float *y, float *p,
                          int mode, Scalars *sc, cudaStream_t st);
-// The FP32 iteration's restriction (mode 0) after a product launched with
-// kFinDefer: it adds the product's block sums of p^T q (pqPart, pqN of them)
-// itself, takes alpha from them and counts the iteration in sc->its; its units'
-// sums of ||r||^2 go to rrPart for the coarse solve to add and test.
-void launch_restrict_update_deferred(const RowBoxDev &B, float *u, const float *r_cur,
-                                     float *r_next, const float *p, const float *q, double *g,
-                                     double *zr, double *rrPart, Scalars *sc,
-                                     const float2 *pqPart, int pqN, cudaStream_t st);
+// The FP32 iteration's restriction, after a product launched with kFinDefer: it
+// adds the product's block sums of p^T q (pqPart, pqN of them) itself, takes
+// alpha from them and counts the iteration in sc->its; r' = r - alpha q (to
+// r_next) and u += alpha p on own rows, g and zr of r' as above; its units' sums
+// of ||r'||^2 go to rrPart for the coarse solve to add and test.
+void launch_restrict_update(const RowBoxDev &B, float *u, const float *r_cur, float *r_next,
+                            const float *p, const float *q, double *g, double *zr,
+                            double *rrPart, Scalars *sc, const float2 *pqPart, int pqN,
+                            cudaStream_t st);
 void launch_to_colmajor(int nItems, const int *itemBox, const int *rowStart,
                         const unsigned char *itemB, const long long *srcOff,
                         const int *boxRowPtr, const long long *boxBase, const int *menr,
                         const float *src, float *dst, cudaStream_t st);
 
 // Block sums that the coarse solve adds beside its own work, making the stopping
-// tests on them: values = 1, ||r||^2 (n of them, launch_restrict_update_deferred);
+// tests on them: values = 1, ||r||^2 (n of them, launch_restrict_update);
 // values = 2, ||r||^2 and then r^T y (n of each, launch_update).
 struct ResidualSums {
     const double *part;   // null: the scalars are set already

@@ -12,6 +12,14 @@
 // load the next kernel's factors, bases and matrix stages meanwhile.  The wait
 // is a no-op for a kernel launched without the attribute.
 //
+// The dense inverse (set-up) departs from this: its pivot and panel kernels
+// trigger as their first step, so that a launch independent of them starts
+// beside them, and that one waits only at its end, in one block, so that what
+// follows both follows.  That is sound because the kernels that trigger so are
+// themselves launched without the attribute (all before them is complete when
+// they start), and so is whatever follows the one beside them.  A kernel
+// launched with the attribute must not trigger before its wait.
+//
 // Triggers pay where measured: in the FP32 product, the coarse solve and (up
 // to kTriggerBlocks blocks) the prolongation, 31.8 against 35.3 us per FP32
 // iteration at 12^3 and 50.4 against 52.7 at 32^3.  In the FP32 restriction

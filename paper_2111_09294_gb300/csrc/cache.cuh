@@ -46,6 +46,12 @@ __device__ __forceinline__ float ld_early(const float *a) {
     return v;
 }
 
+__device__ __forceinline__ double ld_early(const double *a) {
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(a) : "memory");
+    return v;
+}
+
 // What an earlier kernel of the run wrote, read after the wait: the ordinary
 // path through L1.  The read-only path (__ldg, or what the compiler makes of a
 // const __restrict__ pointer) is for data that nothing writes while the kernel

@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "cache.cuh"
 #include "internal.h"
 #include "pdl.cuh"
 
@@ -228,7 +229,9 @@ k_inv_panel(DenseBatch B, int k) {
 
 // ---- A_IJ -= C_I A_kJ, J >= I, mirrored into A_JI ----------------------------------
 //
-// Columns [c0, c0 + 16 CB) of tile (I, J).
+// Columns [c0, c0 + 16 CB) of tile (I, J).  Everything is read from L2: the
+// launches beside another kernel do not wait before they work, and it is a wait
+// that would make the finished kernels' writes visible to ordinary loads.
 template <int CB>
 __device__ __forceinline__ void update_tile(const DenseBatch &B, int m, int k, int I, int J,
                                             int cOff) {
@@ -241,23 +244,32 @@ __device__ __forceinline__ void update_tile(const DenseBatch &B, int m, int k, i
     const double *C = panel_of(B, m, k);
     for (int e = threadIdx.x; e < kNB * kNB; e += blockDim.x) {
         const int i = e / kNB, j = e - i * kNB;
-        X[i * kLd + j] = (r0 + i < n && j < nb) ? C[(long long)(r0 + i) * kNB + j] : 0.0;
+        X[i * kLd + j] =
+            (r0 + i < n && j < nb) ? ld_early(C + (long long)(r0 + i) * kNB + j) : 0.0;
     }
     for (int e = threadIdx.x; e < kNB * W; e += blockDim.x) {
         const int i = e / W, j = e - i * W;
-        Y[i * kLd + j] = (i < nb && c0 + j < n) ? *mat_at(B, m, k0 + i, c0 + j) : 0.0;
+        Y[i * kLd + j] = (i < nb && c0 + j < n) ? ld_early(mat_at(B, m, k0 + i, c0 + j)) : 0.0;
     }
     __syncthreads();
     double acc[4][CB] = {};
     tile_mm<CB>(X, Y, nb, acc);
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 4; ++a) {
+        const int i = r0 + ty + 16 * a;
+        double old[CB];
 #pragma unroll
         for (int b = 0; b < CB; ++b) {
-            const int i = r0 + ty + 16 * a, j = c0 + tx + 16 * b;
-            if (i < n && j < n) *mat_at(B, m, i, j) -= acc[a][b];
+            const int j = c0 + tx + 16 * b;
+            old[b] = i < n && j < n ? ld_early(mat_at(B, m, i, j)) : 0.0;
         }
+#pragma unroll
+        for (int b = 0; b < CB; ++b) {
+            const int j = c0 + tx + 16 * b;
+            if (i < n && j < n) *mat_at(B, m, i, j) = old[b] - acc[a][b];
+        }
+    }
     if (I == J) return;
     // the mirrored tile A_JI = A_IJ^T: new values through shared memory so
     // that both stores are row-wise
@@ -269,7 +281,10 @@ __device__ __forceinline__ void update_tile(const DenseBatch &B, int m, int k, i
     __syncthreads();
     for (int e = threadIdx.x; e < kNB * W; e += blockDim.x) {
         const int jj = e / kNB, ii = e - jj * kNB;   // A(c0 + jj, r0 + ii) -= acc(ii, jj)
-        if (c0 + jj < n && r0 + ii < n) *mat_at(B, m, c0 + jj, r0 + ii) -= X[ii * kLd + jj];
+        if (c0 + jj < n && r0 + ii < n) {
+            double *t = mat_at(B, m, c0 + jj, r0 + ii);
+            *t = ld_early(t) - X[ii * kLd + jj];
+        }
     }
 }
 

@@ -81,3 +81,14 @@ def test_read_only_loads_are_of_setup_data():
             # what is only written (y) may be told apart from the rest
             for const, name in re.findall(r"(const )?[\w<>]+ \*__restrict__ (\w+)", params + body):
                 assert not const or name in SETUP, (f, n, name)
+
+
+def test_tiles_beside_another_kernel_are_read_from_l2():
+    # the dense inverse's trailing update runs beside a kernel without waiting
+    # for it before it works: no ordinary load of the matrix or the panel
+    body, = [b for _, n, _, b in functions() if n == "update_tile"]
+    loads = re.sub(r"ld_early\((?:[^()]|\((?:[^()]|\([^()]*\))*\))*\)", "L2", body)
+    assert "mat_at" not in re.sub(r"\*mat_at\([^()]*\) = |double \*t = mat_at\([^()]*\);", "", loads)
+    assert not re.search(r"\bC\[|-=", loads)
+    assert re.findall(r"\*t\b[^;]*;", re.sub(r"double \*t = [^;]*;", "", loads)) == [
+        "*t = L2 - X[ii * kLd + jj];"]

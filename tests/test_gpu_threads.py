@@ -67,3 +67,28 @@ def test_setups_of_few_and_of_many_matrices_at_once():
     assert a == "same", a
     assert isinstance(b, int) and b > 0, b
     E.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_solves_at_once_are_the_solves_alone(prec):
+    # two host threads, a context, a stream and a load each: the same bits
+    from paper_2111_09294_gb300 import Solver
+    P = X.make("cube8_edge")
+    F = [torch.tensor(f, device="cuda") for f in X.load_cases(P, 2, seed=3)]
+    s = Solver.from_problem(P, precision=prec)
+    ref = [s.solve(f) for f in F]
+    s.close()
+
+    def job(f, u, its):
+        def run():
+            s = Solver.from_problem(P, precision=prec)
+            for _ in range(20):
+                v, info = s.solve(f)
+                assert info["iterations"] == its and torch.equal(u, v)
+            s.close()
+            return "same"
+        return run
+
+    torch.cuda.synchronize()
+    out = _together(*[job(f, u, i["iterations"]) for f, (u, i) in zip(F, ref)])
+    assert out == ["same", "same"], out

@@ -129,7 +129,7 @@ __device__ __forceinline__ void batch_finalize(BatchScalars *bs, int m, int fin,
 // while this one is computed.  Stages run across slice boundaries, as in the
 // single product (k_spmv_lean); each row's terms are added in the order of its
 // slots, partial rows by the same tree.  8 columns at 32^3 (1.1M blocks): 41.5
-// us before, 29.9 now.
+// us before, 29.0 now.
 // The warp's copy schedule (LeanWalk of the single product, step numbers in 32
 // bits: a step is 1,280 bytes).
 struct BatchWalk {
@@ -526,7 +526,7 @@ __device__ __forceinline__ void row_times(const float *z, float rn, float *acc) 
 // The unit's rows of Z~ and W~ and its dof map, shared by the columns, are
 // copied into shared memory before the wait for the product (set-up data);
 // four rows' entries of r, q, p and u are in flight at a time.  8 columns at
-// 32^3 (599 units): 30.4 us before, 17.5 now (four blocks
+// 32^3 (599 units): 30.4 us before, 18.0 now (four blocks
 // per SM).
 template <int MB, int M>
 __device__ __forceinline__ bool restrict_b_unit(const RestrictBArgs &a, int unit, float *stage,
@@ -804,7 +804,7 @@ __device__ __forceinline__ void coarse_load_e(const float *Eb, int k, int rLast,
 // blocks find it after the first.  The partial sums are reduced over the lanes,
 // then over the warps in order.  8 columns, k =
 // 3150: 29.9 us before (G staged by each warp in shared memory through bulk
-// copies and barriers), 22.1 now (three blocks of 80 registers per SM; four of 64
+// copies and barriers), 22.2 now (three blocks of 80 registers per SM; four of 64
 // spill, 39).
 template <int MB, int V>
 __device__ __forceinline__ void coarse_b_body(const CoarseBArgs &a, int blk, int nblk) {

@@ -624,7 +624,7 @@ __device__ __forceinline__ bool restrict_update_unit(const RowBoxDev &B, int uni
 //
 // Bound by latency: 51 MB at 48^3, most of it from L2, between two grid-wide
 // dependencies.  48^3 (543 units): 28.8 us before (dependent loads after the
-// wait, every warp dividing in FP64, a reduction across the blocks), 22.5 now;
+// wait, every warp dividing in FP64, a reduction across the blocks), 22.1 now;
 // 12^3 (11 units): 19.8 before, 12.3 now.
 template <bool YV, bool FEW>
 __global__ void __launch_bounds__(kRowThreads, FEW ? 1 : 4)

@@ -22,7 +22,7 @@
 // triggers the dependent launch of the first part of those tiles as it starts
 // (and takes an SM to itself, by its shared memory, while there are few
 // matrices), the panel of the second part.  k = 3150: 51.8 ms before (the
-// steps' launches one after another, 0.36 ms per pivot block), 37.4 now; k =
+// steps' launches one after another, 0.36 ms per pivot block), 36.8 now; k =
 // 426: 3.4 before, 2.3 now.
 #include <algorithm>
 #include <climits>
